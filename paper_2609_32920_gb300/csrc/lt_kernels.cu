@@ -433,6 +433,28 @@ struct ChainState {
   bool refl;
 };
 
+// Primitives the path hit at its vertices, so that a replay intersects the known primitive
+// instead of searching the scene: the same test on the same primitive gives the hit bit for
+// bit.  HitLog: a lane's own record of the walk it is on; TapeHits: the naive tape's.
+struct HitLog {
+  int prim[kMaxDepth];
+  __device__ __forceinline__ int operator()(int k) const { return prim[k]; }
+};
+struct TapeHits {
+  const float4* tape;
+  int64_t n, p;
+  __device__ __forceinline__ int operator()(int k) const {
+    return __float_as_int(__ldg(&tape[2 * ((size_t)k * n + p)].x)) & 0xffffff;
+  }
+};
+// The hit of a ray on a primitive it is known to meet.
+__device__ __forceinline__ HitRec hit_known(const DevScene& S, float3 org, float3 dir, int prim) {
+  HitRec h;
+  const Prim P = load_prim(S, prim);
+  h.prim = hit_prim(P.o, P.e1, P.e2, P.is_tri, org, dir, h.t, h.b1, h.b2) ? prim : -1;
+  return h;
+}
+
 // Vertex states of the chains the forward walk has just passed through, so that a chain's
 // reverse sweep reads them instead of replaying the chain (its traces run on the few lanes
 // that finish a chain at that step).  Two records, the current chain and the one before
@@ -483,14 +505,14 @@ struct ChainCache {
   }
 };
 
-// Replay the chain from its start to vertex j (a <= j) and trace the ray leaving j.  The
+// Replay the chain from its start to vertex j (a <= j) along the primitives the walk hit.  The
 // chain's first direction is the one the walk sampled at the anchor (the emitter's
 // cosine sample, or the diffuse anchor's, on the side of its normal that faces the chain
 // start), recomputed from the same Philox numbers, so the replay repeats the walk's
-// arithmetic exactly; normalize(x_a - x_p) differs from it in the last bits, which can
-// send a grazing ray to another triangle.
+// arithmetic exactly; normalize(x_a - x_p) differs from it in the last bits.
+template <class H>
 __device__ __forceinline__ bool chain_replay(const DevScene& S, const KParams& kp, uint64_t n, const ChainInfo& c,
-                                             int j, ChainState& st, HitRec& next) {
+                                             int j, ChainState& st, const H& hits) {
   Prim Pa = load_prim(S, c.prim_a);
   float3 x = Pa.o + Pa.e1 * c.ba1 + Pa.e2 * c.ba2;
   float3 din;
@@ -510,13 +532,12 @@ __device__ __forceinline__ bool chain_replay(const DevScene& S, const KParams& k
     Dielectric D = dielectric(din, normalize(nraw), __ldg(S.mat_ior + P.mat));
     float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
     bool refl = D.tir || r.z < D.F;
-    float3 dout = refl ? D.refl : D.refr;
-    HitRec h = trace_closest(S, x, dout, prim);
     if (k == j) {
       st.prim = prim; st.x = x; st.din = din; st.nraw = nraw; st.D = D; st.refl = refl;
-      next = h;
-      return h.prim >= 0;
+      return true;
     }
+    float3 dout = refl ? D.refl : D.refr;
+    HitRec h = hit_known(S, x, dout, hits(k + 1));
     if (h.prim < 0) return false;
     x = x + dout * h.t;
     din = dout;
@@ -569,12 +590,15 @@ __device__ __forceinline__ void spec_adjoint(const ChainState& s, float3 gdout, 
 
 // Reverse-mode sweep back through a chain ending at sliding vertex kt whose position
 // adjoint is gx_t: vertex states come from the forward walk's chain cache when it holds the
-// chain, else they are replayed from the chain start (constant memory, c(c+1)/2 traces for
-// c specular vertices).  Scatters into the height gradient the contributions of every
-// primitive the chain touches and returns the adjoint of the anchor position (through the
-// chain start's incoming direction).
+// chain, else they are replayed from the chain start along the known primitives (constant
+// memory, c(c+1)/2 vertex evaluations and no traversal for c specular vertices; replaying by
+// tracing made a chain of 10 a serial 55-ray tail that the whole launch waited for).  Scatters
+// into the height gradient the contributions of every primitive the chain touches and returns
+// the adjoint of the anchor position (through the chain start's incoming direction).
+template <class H>
 __device__ __forceinline__ float3 chain_reverse(const DevScene& S, const KParams& kp, uint64_t n, const ChainInfo& c,
-                                             int kt, float3 gx_t, float* dh, const ChainCache* cc, int prim_t) {
+                                             int kt, float3 gx_t, float* dh, const ChainCache* cc, int prim_t,
+                                             const H& hits) {
   const ChainRec* rec = nullptr;
   if (cc)
     for (int b = 0; b < 2; ++b)
@@ -594,9 +618,8 @@ __device__ __forceinline__ float3 chain_reverse(const DevScene& S, const KParams
       s.refl = (rec->refl >> i) & 1u;
       hprim = j + 1 < kt ? rec->prim[i + 1] : prim_t;
     } else {
-      HitRec h;
-      if (!chain_replay(S, kp, n, c, j, s, h)) { set_err(S, ERR_BOUNDS); return f3(0, 0, 0); }
-      hprim = h.prim;
+      if (!chain_replay(S, kp, n, c, j, s, hits)) { set_err(S, ERR_BOUNDS); return f3(0, 0, 0); }
+      hprim = j + 1 < kt ? hits(j + 1) : prim_t;
     }
     Prim Q = load_prim(S, hprim);
     float3 m = cross(Q.e1, Q.e2);
@@ -630,11 +653,12 @@ __device__ __forceinline__ float3 chain_reverse(const DevScene& S, const KParams
   return f3(0, 0, 0);
 }
 
-// Geometry-only replay of the path from the emitter up to vertex `target`; returns the
-// chain that vertex ends (valid when it is a sliding diffuse vertex).  Used to recover
-// an earlier chain when a position adjoint has to continue through it.
+// Geometry-only replay of the path from the emitter up to vertex `target` along the known
+// primitives; returns the chain that vertex ends (valid when it is a sliding diffuse vertex).
+// Used to recover an earlier chain when a position adjoint has to continue through it.
+template <class H>
 __device__ __noinline__ bool replay_chain_of(const DevScene& S, const KParams& kp, uint64_t n, int target,
-                                            ChainInfo& out) {
+                                            ChainInfo& out, const H& hits) {
   Walk w;
   float3 x0;
   walk_start(S, kp.seed, n, f3(1, 1, 1), w, x0);
@@ -644,7 +668,7 @@ __device__ __noinline__ bool replay_chain_of(const DevScene& S, const KParams& k
   ch.ka = -1;
   for (int k = 0; k <= target; ++k) {
     Vtx v;
-    if (!walk_hit(S, w, v)) return false;
+    if (!walk_finish(S, w, hit_known(S, w.org, w.dir, hits(k)), v)) return false;
     if (v.attached && !v.diffuse) ch = chain_at(an, k, v, 0.0f);
     if (k == target) {
       out = ch;
@@ -665,10 +689,11 @@ __device__ __noinline__ bool replay_chain_of(const DevScene& S, const KParams& k
 // Propagate a position adjoint on the sliding end kt of chain c back to the parameters,
 // continuing through earlier chains while the anchor is itself sliding (those chains'
 // Fresnel factors were already counted, so they are re-traversed with zero weight).
+template <class H>
 __device__ __forceinline__ void propagate_sliding(const DevScene& S, const KParams& kp, uint64_t n, ChainInfo c, int kt,
-                                               float3 gx, float* dh, const ChainCache* cc, int prim_t) {
+                                               float3 gx, float* dh, const ChainCache* cc, int prim_t, const H& hits) {
   for (int guard = 0; guard < kMaxDepth; ++guard) {
-    float3 g_anchor = chain_reverse(S, kp, n, c, kt, gx, dh, cc, prim_t);
+    float3 g_anchor = chain_reverse(S, kp, n, c, kt, gx, dh, cc, prim_t, hits);
     if (c.kanchor < 0) return;  // the emitter does not move
     if (!c.anchor_sliding) {
       scatter_heights(S, dh, c.prim_p, c.bp1, c.bp2, g_anchor, f3(0, 0, 0));
@@ -683,7 +708,7 @@ __device__ __forceinline__ void propagate_sliding(const DevScene& S, const KPara
           prev.lam = 0.0f;  // geometry only, as in the replay: its Fresnel factors are counted
           found = true;
         }
-    if (!found && !replay_chain_of(S, kp, n, c.kanchor, prev)) { set_err(S, ERR_BOUNDS); return; }
+    if (!found && !replay_chain_of(S, kp, n, c.kanchor, prev, hits)) { set_err(S, ERR_BOUNDS); return; }
     prim_t = c.prim_p;
     kt = c.kanchor;
     gx = g_anchor;
@@ -716,15 +741,15 @@ __device__ __forceinline__ float3 tex_pos_adjoint(const float* albedo, int4 m, c
 
 // Flush a vertex's completed adjoint: attached vertices map through their surface
 // coordinates, sliding ones run the chain's reverse sweep (their normal is explicit).
-template <bool CH>
+template <bool CH, class H>
 __device__ __forceinline__ void pend_flush(const DevScene& S, const KParams& kp, uint64_t n, const PendAdj& p,
-                                           float* dh, const ChainCache* cc) {
+                                           float* dh, const ChainCache* cc, const H& hits) {
   if (!dh || p.prim < 0) return;
   if (!CH || !p.sliding) {
     scatter_heights(S, dh, p.prim, p.b1, p.b2, p.gx, p.gn);
   } else {
     scatter_heights(S, dh, p.prim, 0.0f, 0.0f, f3(0, 0, 0), p.gn);
-    propagate_sliding(S, kp, n, p.chain, p.k, p.gx, dh, cc, p.prim);
+    propagate_sliding(S, kp, n, p.chain, p.k, p.gx, dh, cc, p.prim, hits);
   }
 }
 
@@ -733,15 +758,15 @@ __device__ __forceinline__ void pend_flush(const DevScene& S, const KParams& kp,
 // specular vertex starts a chain (its Fresnel factors weigh lam_chain); a non-specular
 // vertex becomes the new pending anchor (sliding when it ends a chain).
 // CH = false compiles the variant for scenes without dielectrics (no chains exist).
-template <bool CH>
+template <bool CH, class H>
 __device__ __forceinline__ void att_enter(const DevScene& S, const KParams& kp, uint64_t n, int k, const Vtx& v,
                                           float lam_seg, float lam_chain, PendAdj& pv, ChainInfo& chain,
-                                          float* dh, const ChainCache* cc) {
+                                          float* dh, const ChainCache* cc, const H& hits) {
   if (!CH || v.attached) {
     PendAdj cur;
     pend_init(cur, v.prim, k, v.b1, v.b2, v.x, v.nraw);
     seg_adjoint(pv.x, pv.nr, v.x, v.nraw, lam_seg, pv.gx, pv.gn, cur.gx, cur.gn);
-    pend_flush<CH>(S, kp, n, pv, dh, cc);
+    pend_flush<CH>(S, kp, n, pv, dh, cc, hits);
     if (CH && !v.diffuse) {
       chain = chain_at(pv, k, v, lam_chain);
       scatter_heights(S, dh, v.prim, v.b1, v.b2, cur.gx, cur.gn);
@@ -1291,6 +1316,10 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   pv.prim = -1;
   ChainCache cc;
   cc.reset();
+  // primitives of the lane's path: pass 3 of the fused form replays along those of pass 2, and
+  // a chain's reverse sweep along those of the walk it ends
+  constexpr bool LOG = CH || MODE == 0;
+  HitLog log;
   TravState ts;  // the lane's ray in flight (see TravState)
   LocalStack stk;
   bool inflight = false;
@@ -1354,7 +1383,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         const unsigned busy = __ballot_sync(0xffffffffu, phase == PASS2 || phase == PASS3 || (more && phase == IDLE));
         if (__popc(fq) >= kFlushBatch || busy == 0u) {
           if (phase == FLUSH) {
-            pend_flush<CH>(S0, kp0, (uint64_t)(kp0.path_offset + p), pv, gs.d_heights, &cc);
+            pend_flush<CH>(S0, kp0, (uint64_t)(kp0.path_offset + p), pv, gs.d_heights, &cc, log);
             phase = IDLE;
           }
         }
@@ -1395,7 +1424,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     HitRec h;
     h.prim = -1;
     bool pending = false;  // the ray has visits left: the lane resumes it in the next step
-    if constexpr (CH) {
+    if (MODE == 0 && trav && phase == PASS3) {
+      h = hit_known(S, w.org, w.dir, log(k));
+    } else if constexpr (CH) {
       // the specular-chain variants keep whole traversals: the resumable state would
       // push them past the register budget that their chain transport needs
       if (trav) h = trace_closest<ST>(S, w.org, w.dir, w.skip, &cs);
@@ -1407,6 +1438,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     }
     Vtx v;
     const bool alive = trav && !pending && walk_finish(S, w, h, v);
+    if (LOG && alive) log.prim[k] = v.prim;
     float3 ns = f3(0, 0, 0);
     Conn c;
     c.valid = false; c.ux = c.uy = 0.0f;
@@ -1476,7 +1508,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
         // attached segment weight and chain bookkeeping: every connection from here on
         // carries this vertex's factors, so they weigh the remaining adjoint before Eq. 16
-        if (att) att_enter<CH>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc);
+        if (att) att_enter<CH>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc, log);
         const bool rec_chain = CH && att && !v.diffuse;
         if (rec_chain) cc.record(chain, k, v, w.dir);
         float3 rho = f3(0, 0, 0);
@@ -1507,7 +1539,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         if (DEFER && pv.prim >= 0 && pv.sliding && g.d_heights) {
           phase = FLUSH;
         } else {
-          if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc);
+          if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc, log);
           phase = IDLE;
         }
       }
@@ -1667,6 +1699,7 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
   pv.prim = -1;
   ChainCache cc;
   cc.reset();
+  HitLog log;  // primitives of the lane's path, for the chain sweeps
   TravState ts;
   LocalStack stk;
   bool inflight = false;
@@ -1739,7 +1772,8 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
       continue;
     }
     const float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
-    if (att) att_enter<CH>(S, kp, n, k, v, lam, lam, pv, chain, g.d_heights, &cc);
+    if (CH) log.prim[k] = v.prim;
+    if (att) att_enter<CH>(S, kp, n, k, v, lam, lam, pv, chain, g.d_heights, &cc, log);
     const bool rec_chain = CH && att && !v.diffuse;
     if (rec_chain) cc.record(chain, k, v, w.dir);
     float3 ns = f3(0, 0, 0), rho = f3(0, 0, 0);
@@ -1757,7 +1791,7 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     if (rec_chain) cc.record_branch(refl);
     walk_rr(kp, n, k, w);
     if (++k > R) {
-      if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc);
+      if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc, log);
       busy = false;
     }
   }
@@ -1908,7 +1942,7 @@ __global__ void __launch_bounds__(128) k_naive(DevScene S, KParams kp, const flo
             c.anchor_sliding = !((((uint32_t)__float_as_int(sp.x)) >> 24) & 16u);
           }
           scatter_heights(S, g.d_heights, prim, 0.0f, 0.0f, f3(0, 0, 0), gn);
-          propagate_sliding(S, kp, n, c, k, gx, g.d_heights, nullptr, prim);
+          propagate_sliding(S, kp, n, c, k, gx, g.d_heights, nullptr, prim, TapeHits{tape, kp.n_paths, p});
         }
       }
       acc = acc + P3;
@@ -1960,9 +1994,11 @@ __global__ void __launch_bounds__(128) k_bidir_light(DevScene S, KParams kp, Bid
     float pf0 = 0.0f;
     float3 dtot = f3(0, 0, 0);
     uint64_t valid = 0;
+    HitLog log;  // primitives of the path: the adjoint's second walk replays along them
     for (int k = 0; k < kp.max_depth; ++k) {
       Vtx v;
       if (!walk_hit(S, w, v)) break;
+      if (BWD) log.prim[k] = v.prim;
       if (k == 0) {
         const float3 d = v.x - x0;
         pf0 = fabsf(dot(S.ln, w.dir)) * fabsf(dot(v.n, w.dir)) / (kPi * dot(d, d));
@@ -1997,7 +2033,8 @@ __global__ void __launch_bounds__(128) k_bidir_light(DevScene S, KParams kp, Bid
     const int last = 63 - __clzll((long long)valid);
     for (int k = 0; k <= last; ++k) {
       Vtx v;
-      if (!walk_hit(S, w, v)) { set_err(S, ERR_BOUNDS); break; }  // the replay must reach `last`
+      // the replay must reach `last`
+      if (!walk_finish(S, w, hit_known(S, w.org, w.dir, log(k)), v)) { set_err(S, ERR_BOUNDS); break; }
       if (k == 0) {
         const float3 d = v.x - x0;
         pf0 = fabsf(dot(S.ln, w.dir)) * fabsf(dot(v.n, w.dir)) / (kPi * dot(d, d));
@@ -2047,12 +2084,15 @@ __device__ __forceinline__ void cam_start(const DevScene& S, const KParams& kp, 
   cw.thr = f3(1, 1, 1);
   cw.geo1 = cw.pfilm = 0.0f;
 }
+// VIS: the first walk (searches the scene and tests visibility); else a replay along the known
+// primitive `prim` with the known visibility.
 template <bool VIS>
 __device__ __forceinline__ bool cam_vertex(const DevScene& S, const KParams& kp, const BidirArgs& ba, uint64_t c,
                                            int m, CamWalk& cw, bool nee_known, float3& contrib, bool& nee,
-                                           TexFoot* foot, float3& rho, uint32_t& hash) {
-  const HitRec h = trace_closest(S, cw.org, cw.dir, cw.skip);
+                                           TexFoot* foot, float3& rho, uint32_t& hash, int& prim) {
+  const HitRec h = VIS ? trace_closest(S, cw.org, cw.dir, cw.skip) : hit_known(S, cw.org, cw.dir, prim);
   if (h.prim < 0) return false;
+  if (VIS) prim = h.prim;
   const Prim P = load_prim(S, h.prim);
   const int4 mt = __ldg(S.mat + P.mat);
   if (mt.x != MAT_DIFFUSE) return false;  // the emitter absorbs (seen directly it is black)
@@ -2111,8 +2151,11 @@ __global__ void __launch_bounds__(128) k_bidir_cam(DevScene S, KParams kp, Bidir
     float3 total = f3(0, 0, 0), contrib, rho;
     uint64_t nees = 0;
     bool nee;
+    HitLog log;  // primitives of the sample, for the replay
     for (int m = 1; m <= kp.max_depth; ++m) {
-      if (!cam_vertex<true>(S, kp, ba, (uint64_t)c, m, cw, false, contrib, nee, nullptr, rho, hash)) break;
+      int prim;
+      if (!cam_vertex<true>(S, kp, ba, (uint64_t)c, m, cw, false, contrib, nee, nullptr, rho, hash, prim)) break;
+      if (BWD) log.prim[m - 1] = prim;
       total = total + contrib;
       if (nee) nees |= 1ull << (m - 1);
     }
@@ -2130,8 +2173,9 @@ __global__ void __launch_bounds__(128) k_bidir_cam(DevScene S, KParams kp, Bidir
     const int last = 64 - __clzll((long long)nees);
     for (int m = 1; m <= last; ++m) {
       TexFoot foot;
+      int prim = log(m - 1);
       if (!cam_vertex<false>(S, kp, ba, (uint64_t)c, m, cw, (nees >> (m - 1)) & 1ull, contrib, nee, &foot, rho,
-                             hash)) {
+                             hash, prim)) {
         set_err(S, ERR_BOUNDS);  // the replay must reach the last connection
         break;
       }
@@ -2492,9 +2536,11 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
     float Apos[4] = {0, 0, 0, 0};
     LitV pa = em, pb = em;  // vertices k-2 and k-1
     bool singular = false;
+    HitLog log;  // primitives of the path: pass 3 replays along them
     for (int k = 0; k < kp.max_depth; ++k) {
       Vtx v;
       if (!walk_hit(S, w, v)) break;
+      log.prim[k] = v.prim;
       const LitV cur = {v.prim, v.b1, v.b2, !v.diffuse, false};
       if (k >= 1) lit_advance(S, kp, n, k, pa, pb, v.prim, Jacc, singular);
       const float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
@@ -2538,7 +2584,8 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
     singular = false;
     for (int k = 0; k <= last; ++k) {
       Vtx v;
-      if (!walk_hit(S, w, v)) { set_err(S, ERR_BOUNDS); break; }  // the replay must reach `last`
+      // the replay must reach `last`
+      if (w.dead || !walk_finish(S, w, hit_known(S, w.org, w.dir, log(k)), v)) { set_err(S, ERR_BOUNDS); break; }
       const LitV cur = {v.prim, v.b1, v.b2, !v.diffuse, false};
       if (k >= 1) {
         lit_advance(S, kp, n, k, pa, pb, v.prim, Jacc, singular);
@@ -2549,7 +2596,7 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
         }
       }
       const float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
-      att_enter<true>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc);
+      att_enter<true>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc, log);
       const bool rec_chain = !v.diffuse;
       if (rec_chain) cc.record(chain, k, v, w.dir);
       float3 ns = f3(0, 0, 0), rho = f3(0, 0, 0);
@@ -2588,7 +2635,7 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
       pb = cur;
       pb.refl = refl;
     }
-    pend_flush<true>(S, kp, n, pv, g.d_heights, &cc);
+    pend_flush<true>(S, kp, n, pv, g.d_heights, &cc, log);
   }
   sink_end(kp, g0, sgrad);
   block_add3(g0.d_Le, gLe);
