@@ -124,17 +124,21 @@ typedef struct {
   size_t lrb3_state_bytes; /* size of lrb3_state                                    */
   int lrb3_mask_ready;  /* lt_primal(LT_EST_PLAIN) given lrb3_state also stores each
                            path's connection-validity mask there, the list of the
-                           paths that have a valid connection, and each path's first
-                           valid connection (film position, contribution).  Set 1 in
-                           the opts of lt_backward_lrb3 when that primal ran with the
-                           same seed, paths, depth, scene and parameters: pass 2 then
-                           takes validity from the mask, traces no visibility rays,
-                           stops each path after its last valid connection, forms
-                           delta_total of a path with one valid connection from the
-                           stored connection without replaying it, and passes 2 and 3
-                           visit only the listed paths (the others have delta_total
-                           zero; their stored colour words and path_dbg rows are left
-                           as they are and not read).                           */
+                           paths that have a valid connection, and a record of each
+                           listed path: the primitives its first vertices hit, and
+                           the connection (film position, contribution) of a path
+                           with one.  Set 1 in the opts of lt_backward_lrb3 when that
+                           primal ran with the same seed, paths, depth, scene and
+                           parameters: pass 2 then takes validity from the mask,
+                           traces no visibility rays, stops each path after its last
+                           valid connection, forms delta_total of a path with one
+                           valid connection from the stored connection without
+                           replaying it, passes 2 and 3 visit only the listed paths
+                           (the others have delta_total zero; their records and
+                           path_dbg rows are left as they are and not read), and
+                           their replays intersect the recorded primitive at a
+                           path's first vertices instead of searching the scene
+                           (the same hit bit for bit).                          */
   int rr_depth;         /* Russian roulette: after each vertex of depth >= rr_depth a
                            path continues with probability rr_prob (Philox stream 2
                            of that depth) and its throughput is divided by rr_prob;
@@ -465,7 +469,8 @@ lt_status lt_bidir_backward(lt_scene* scene, const lt_params* params, const lt_r
  * vertex's splat record (film position and contribution L_i, 20 B per vertex, memory
  * linear in max_depth) in `buffer`; this call computes delta_total = sum_i Lbar_i * L_i
  * from those records without tracing (Eq. 14) and then replays each path once to
- * backpropagate (Eq. 15-17), so two traversals in all instead of LRB-3's three.  Same
+ * backpropagate (Eq. 15-17), intersecting the primitives of its first vertices that the primal
+ * kept (160 bits of a 40 B per-path record) and searching the scene beyond them.  Same
  * result as lt_backward_lrb3.  buffer: DEVICE, lt_lrb2_buffer_bytes(opts) bytes, written
  * by lt_primal(LT_EST_BUFFERED) with the same opts (LT_ERR_OOM if smaller).  path_dbg
  * (optional) [n_paths][4] = (delta_total rgb, n valid connections). */
@@ -474,15 +479,15 @@ lt_status lt_backward_lrb2(lt_scene* scene, const lt_params* params, const lt_re
                            void* stream);
 size_t lt_lrb2_buffer_bytes(const lt_render_opts* opts);
 
-/* Bytes of the optional LRB-3 per-path state (opts->lrb3_state): 16 B (delta_total rgb,
- * validity bits 0-31), 4 B (validity bits 32-63) and 4 B (the list of paths with a valid
- * connection) per path, then the list's length and the passes' counters (256 B), then
- * 20 B per path (film position and contribution of the path's first valid connection,
- * written by the plain primal: pass 2 takes delta_total of a path with exactly one valid
- * connection from it instead of replaying the path), then 4 B per path and a fixed 4.2 MB
- * (the order in which the plain primal takes the paths, sorted by the cell of each path's
- * first direction, and the counting sort's work area; the order changes no result); each
- * array 256-B aligned. */
+/* Bytes of the optional LRB-3 per-path state (opts->lrb3_state): a record of 32 B per path
+ * (delta_total rgb; the primitives that the path's first vertices hit, as many as fit in 256
+ * bits for pass 2 and in 160 for pass 3; for a path with exactly one valid connection its film
+ * position and contribution, from which pass 2 takes delta_total instead of replaying the
+ * path, and 96 bits of primitives), 8 B of validity bits and 4 B (the list of paths with a
+ * valid connection) per path, the list's length and the passes' counters (256 B), then 4 B
+ * per path and a fixed 4.2 MB (the order in which the plain primal takes the paths, sorted by
+ * the cell of each path's first direction, and the counting sort's work area; the order
+ * changes no result): 48 B per path and 4.2 MB, flat in depth; each array 256-B aligned. */
 size_t lt_lrb3_state_bytes(const lt_render_opts* opts);
 
 /* Bytes of one ResLRB record (constant per path). */

@@ -359,13 +359,21 @@ KParams kparams(const lt_params* p, const lt_render_opts* o) {
   k.list = nullptr;
   k.list_n = nullptr;
   k.ticket = nullptr;
-  k.conn1 = nullptr;
-  k.conn1z = nullptr;
+  k.multi = nullptr;
+  k.multi_n = nullptr;
+  k.hits = HitBits{0, 0, 0, 0};
   k.order = nullptr;
   k.jac_noise = o->jac_noise;
   k.noise_seed = o->noise_seed;
   k.det_eps = o->det_eps > 0.0f ? o->det_eps : 1e-6f;
   return k;
+}
+
+// Primitives kept in the per-path records of a scene: as many bits as its largest index needs.
+HitBits hit_bits(const lt_scene* s) {
+  int b = 1;
+  while (b < 31 && (1ll << b) < s->n_prims) ++b;
+  return HitBits{b, std::min(256 / b, kMaxDepth), std::min(160 / b, kMaxDepth), std::min(96 / b, kMaxDepth)};
 }
 
 // Gradients accumulate per block in shared memory for each parameter array that fits in
@@ -803,8 +811,7 @@ lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, in
   KParams kp = kparams(p, o);
   if (est == LT_EST_PLAIN && o->lrb3_state) {
     kp.vstate = o->lrb3_state;
-    kp.conn1 = (float4*)((char*)o->lrb3_state + lrb3_state_conn4(o->n_paths));
-    kp.conn1z = (float*)((char*)o->lrb3_state + lrb3_state_connz(o->n_paths));
+    kp.hits = hit_bits(s);
     if (o->n_paths <= kListMaxPaths) {
       // the list of the paths with a valid connection, for LRB-3 passes 2 and 3
       char* base = (char*)o->lrb3_state;
@@ -826,6 +833,7 @@ lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, in
       kp.order = order;
     }
   }
+  if (est == LT_EST_BUFFERED) kp.hits = hit_bits(s);
   cudaError_t e = launch_primal(dev_for(s, o), kp, est, image, aux, cfg_for(s, o), st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_primal: ") + cudaGetErrorString(e));
   return LT_OK;
@@ -851,19 +859,18 @@ lt_status lt_backward_lrb3(lt_scene* s, const lt_params* p, const lt_render_opts
     if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb3: ") + cudaGetErrorString(e));
     return LT_OK;
   }
-  if (o->lrb3_state && o->lrb3_mask_ready) {
-    // the primal recorded each path's first valid connection: pass 2 takes delta_total of a
-    // path with one valid connection from it
-    kp.conn1 = (float4*)((char*)o->lrb3_state + lrb3_state_conn4(o->n_paths));
-    kp.conn1z = (float*)((char*)o->lrb3_state + lrb3_state_connz(o->n_paths));
-  }
+  // the primal recorded the primitives of each path's first vertices and, for a path with one
+  // valid connection, that connection
+  if (o->lrb3_state && o->lrb3_mask_ready) kp.hits = hit_bits(s);
   if (o->lrb3_state && o->lrb3_mask_ready && o->n_paths <= kListMaxPaths) {
     // the primal listed the paths with a valid connection: passes 2 and 3 visit only those
     char* base = (char*)o->lrb3_state;
     kp.list = (uint32_t*)(base + lrb3_state_list(o->n_paths));
     kp.list_n = (unsigned long long*)(base + lrb3_state_count(o->n_paths));
     kp.ticket = kp.list_n + 1;
-    LT_CUDA(cudaMemsetAsync(kp.ticket, 0, 2 * sizeof(unsigned long long), st));
+    kp.multi_n = kp.list_n + 3;
+    kp.multi = (uint32_t*)(base + lrb3_state_order(o->n_paths));
+    LT_CUDA(cudaMemsetAsync(kp.ticket, 0, 3 * sizeof(unsigned long long), st));
   }
   cudaError_t e = launch_lrb3(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, gp,
                               o->lrb3_state, o->lrb3_state && o->lrb3_mask_ready, cfg_for(s, o), st);
@@ -902,6 +909,8 @@ lt_status lt_backward_lrb2(lt_scene* s, const lt_params* p, const lt_render_opts
   if (o->n_paths == 0) return LT_OK;
   KParams kp = kparams(p, o);
   set_privatization(s, g, kp, o->scatter);
+  kp.hits = hit_bits(s);
+  kp.hits.cap1 = kp.hits.cap3;  // every record of the buffer has the wide form
   cudaError_t e = launch_lrb2(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, buf, gp,
                               cfg_for(s, o), st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb2: ") + cudaGetErrorString(e));
@@ -1336,7 +1345,9 @@ lt_status lt_batch_create(const lt_batch_item* items, int n, void* stream, lt_ba
     J.image = it.image;
     J.rec = it.records;
     J.state = it.opts.lrb3_state;
-    J.kp.vstate = it.opts.lrb3_state;  // the batched plain primal stores validity masks there
+    // the batched plain primal stores validity masks and hits there
+    J.kp.vstate = it.opts.lrb3_state;
+    if (it.opts.lrb3_state && b->mask_ready) J.kp.hits = hit_bits(it.scene);
     set_privatization(it.scene, &it.grads, J.kp);  // used by pass 3 over spans only
     b->span_smem = std::max(b->span_smem, sizeof(float) * (size_t)J.kp.priv_n);
     J.att = it.opts.attached != 0;

@@ -447,6 +447,38 @@ struct TapeHits {
     return __float_as_int(__ldg(&tape[2 * ((size_t)k * n + p)].x)) & 0xffffff;
   }
 };
+// Primitives packed `bits` each into consecutive words (see HitBits), appended in vertex order:
+// the current word is in a register, full ones in the lane's local memory.
+struct HitPack {
+  uint32_t w[8];
+  uint32_t acc;
+  __device__ __forceinline__ void put(const HitBits& hb, int k, int prim) {
+    if (k >= hb.cap) return;
+    const int off = k * hb.bits, sh = off & 31;
+    if (sh == 0) acc = 0u;
+    acc |= (uint32_t)prim << sh;
+    if (sh + hb.bits >= 32) {
+      w[off >> 5] = acc;
+      acc = sh + hb.bits > 32 ? (uint32_t)prim >> (32 - sh) : 0u;
+    }
+  }
+  // after the last of n vertices
+  __device__ __forceinline__ void close(const HitBits& hb, int n) {
+    const int off = min(n, hb.cap) * hb.bits;
+    if (off & 31) w[off >> 5] = acc;
+  }
+};
+// ... and read back at any vertex below the record's capacity.  The result is clamped to the
+// scene's primitives, so that a state the primal did not fill cannot address beyond them.
+template <int W>
+struct HitWords {
+  uint32_t w[W + 1];
+  __device__ __forceinline__ int get(const HitBits& hb, int k, int n_prims) const {
+    const int off = k * hb.bits;
+    const uint32_t v = __funnelshift_r(w[off >> 5], w[(off >> 5) + 1], off & 31);
+    return min((int)(v & ((1u << hb.bits) - 1u)), n_prims - 1);
+  }
+};
 // The hit of a ray on a primitive it is known to meet.
 __device__ __forceinline__ HitRec hit_known(const DevScene& S, float3 org, float3 dir, int prim) {
   HitRec h;
@@ -463,6 +495,9 @@ __device__ __forceinline__ HitRec hit_known(const DevScene& S, float3 org, float
 // states are the ones the replay would compute, from the same arithmetic.
 constexpr int kChainCache = 4;
 constexpr int kDraws = 4;  // path draws per lane and step of the LRB-3 loop
+// lanes of a warp beyond their recorded hits that search together (box pass 3: 1 6.04 ms, 6 4.65,
+// 12 4.55, 20 5.16)
+constexpr int kSearchBatch = 12;
 constexpr int kFlushBatch = 16;  // waiting lanes of a warp that sweep their chains together (swept 8-24)
 struct ChainRec {
   ChainInfo info;
@@ -979,8 +1014,10 @@ __device__ __forceinline__ void add3(float* d, float3 v) {
 // belongs to (BatchDispenser); S0, kp0, image0 and aux0 are not used.
 // LEARN compiles the learned reservoir target (ResLRB only); plain ResLRB does not carry its
 // registers.  ST compiles the work census (rays, box and primitive tests, vertices,
-// connections) of a counting variant.  AGG compiles warp-aggregated splat atomics.
-template <int EST, bool BATCH, bool LEARN = false, bool ST = false, bool AGG = false>
+// connections) of a counting variant.  AGG compiles warp-aggregated splat atomics.  REC compiles
+// the plain estimator's LRB-3 state (masks, list, records; without it k_primal<0, false> renders
+// 1.5 M paths of the box in 3.3 ms, with it in 3.45 ms).
+template <int EST, bool BATCH, bool LEARN = false, bool ST = false, bool AGG = false, bool REC = EST == 0>
 __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& kp0, float* __restrict__ image0,
                                             void* aux0, const BatchArgs& ba) {
   // learned reservoir target: network image, one 32x16 feature tile per warp, and two
@@ -1003,7 +1040,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
   // the plain estimator given the LRB-3 state takes 32-path chunks from a counter shared by
   // the grid (no warp waits for a slower one at the end); the others split the range statically
   if (BATCH) bdisp.init();
-  else if (EST == 0 && kp0.ticket) disp.init_dynamic(kp0.n_paths, kp0.ticket);
+  else if (REC && kp0.ticket) disp.init_dynamic(kp0.n_paths, kp0.ticket);
   else disp.init(kp0.n_paths);
   int jb = 0;
   bool busy = false, more = true, active = false;
@@ -1021,6 +1058,9 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
   TravState ts;  // the lane's ray in flight (see TravState)
   LocalStack stk;
   bool inflight = false;
+  // for the per-path record: the primitives hit, and the first valid connection
+  HitPack hp;
+  float c1[5];
   Census cs = {0, 0, 0};
   uint32_t nverts = 0, nconns = 0;
   while (true) {
@@ -1036,7 +1076,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
       if (got < 0) {
         more = false;
       } else {
-        p = (!BATCH && kp0.order) ? (int64_t)kp0.order[got] : got;
+        p = (REC && !BATCH && kp0.order) ? (int64_t)kp0.order[got] : got;
         if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
         active = !kp.mask || kp.mask[p];
         float3 x0;
@@ -1065,7 +1105,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
     }
     Vtx v;
     const bool alive = trav && !pending && walk_finish(S, w, h, v);
-    if (EST == 0 && !BATCH && kp0.list) {
+    if (REC && !BATCH && kp0.list) {
       // a path that ends now with a valid connection joins the list that LRB-3 passes 2
       // and 3 visit (one atomic per warp and step)
       const bool ends = busy && !pending && !alive && active && vmask != 0ull;
@@ -1141,13 +1181,30 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         rec[0] = make_float4(__int_as_float(active ? R : -1), wgt, Rux, Ruy);
         rec[1] = make_float4(Sh.x, Sh.y, Sh.z, 0.0f);
       }
-      if (EST == 0 && kp.vstate) {
-        // the validity mask for LRB-3 pass 2 (bits 0-31 in the w of the float4 record,
-        // bits 32-63 in the uint32 array); the rgb part is pass 2's to write
-        float4* xrec = (float4*)kp.vstate;
-        uint32_t* xhi = (uint32_t*)((char*)kp.vstate + lrb3_state_split(kp.n_paths));
-        reinterpret_cast<float*>(xrec + p)[3] = __uint_as_float((uint32_t)(active ? vmask : 0ull));
-        xhi[p] = (uint32_t)((active ? vmask : 0ull) >> 32);
+      if (REC && kp.vstate) {
+        // the validity mask and, with a valid connection, the record (see lrb3_state_bytes)
+        const PathState ps = path_state(kp.vstate, kp.n_paths);
+        const uint64_t vm = active ? vmask : 0ull;
+        ps.mlo[p] = (uint32_t)vm;
+        ps.mhi[p] = (uint32_t)(vm >> 32);
+        if (vm) {
+          hp.close(kp.hits, k);
+          const bool one = (vm & (vm - 1)) == 0ull;
+          const float4 a = make_float4(__uint_as_float(hp.w[0]), __uint_as_float(hp.w[1]), __uint_as_float(hp.w[2]),
+                                       one ? c1[0] : __uint_as_float(hp.w[3]));
+          const float4 b = one ? make_float4(c1[1], c1[2], c1[3], c1[4])
+                               : make_float4(__uint_as_float(hp.w[4]), __uint_as_float(hp.w[5]),
+                                             __uint_as_float(hp.w[6]), __uint_as_float(hp.w[7]));
+          ps.a[ps.step * p] = a;
+          ps.b[ps.step * p] = b;
+        }
+      }
+      if (EST == 3) {
+        hp.close(kp.hits, k);
+        const PathState ps = lrb2_path_state(aux, kp.n_paths, kp.max_depth);
+        ps.a[ps.step * p] = make_float4(__uint_as_float(hp.w[0]), __uint_as_float(hp.w[1]),
+                                        __uint_as_float(hp.w[2]), __uint_as_float(hp.w[3]));
+        ps.b[ps.step * p].x = __uint_as_float(hp.w[4]);
       }
       if (EST == 2) ((int*)aux)[p] = active ? k : 0;
       if (EST == 3) ((int*)((char*)aux + lrb2_layout(kp.n_paths, kp.max_depth).counts))[p] = active ? k : 0;
@@ -1166,11 +1223,10 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         if (ST) ++nconns;
         ++nconn;
         L = mul(w.beta, rho) * (c.geo * kp.inv_n);
-        if (EST == 0 && !BATCH && kp.conn1 && vmask == 0ull) {
-          // the path's first valid connection: LRB-3 pass 2 takes delta_total from this
-          // record when it stays the only one
-          kp.conn1[p] = make_float4(c.ux, c.uy, L.x, L.y);
-          kp.conn1z[p] = L.z;
+        if (REC && vmask == 0ull) {
+          // the path's first valid connection: LRB-3 pass 2 takes delta_total from its record
+          // when it stays the only one
+          c1[0] = c.ux; c1[1] = c.uy; c1[2] = L.x; c1[3] = L.y; c1[4] = L.z;
         }
         vmask |= 1ull << k;
         if (active) {
@@ -1201,6 +1257,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         }
       }
     }
+    if ((REC && kp.vstate) || EST == 3) hp.put(kp.hits, k, v.prim);
     bool refl = walk_scatter(S, w, v, ns, rho, r);
     walk_rr(kp, n, k, w);
     fnv(hash, (uint32_t)v.P.orig);
@@ -1233,9 +1290,9 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
 // Primal light tracing (Sec. 3.1, Eq. 1-2, splats by Eq. 20) for one estimator: EST 0 plain
 // (with the LRB-3 state: validity masks, path list, first connections), 1 ResLRB reservoir
 // records (Sec. 4.2, Eq. 8-9), 2 naive per-vertex tape (Sec. 3.2), 3 buffered splat records.
-template <int EST>
+template <int EST, bool REC = false>
 __global__ void __launch_bounds__(128) k_primal(DevScene S, KParams kp, float* __restrict__ image, void* aux) {
-  primal_body<EST, false>(S, kp, image, aux, BatchArgs{});
+  primal_body<EST, false, false, false, false, REC>(S, kp, image, aux, BatchArgs{});
 }
 // Plain primal with warp-aggregated splat atomics (opts.scatter 3)
 __global__ void __launch_bounds__(128) k_primal_agg(DevScene S, KParams kp, float* __restrict__ image, void* aux) {
@@ -1257,6 +1314,13 @@ __global__ void __launch_bounds__(256) k_primal_batch(BatchArgs ba) {
   primal_body<EST, true>(ba.jobs[0].S, ba.jobs[0].kp, nullptr, nullptr, ba);
 }
 
+// delta_total of a path with one valid connection from its record (see lrb3_state_bytes).
+__device__ __forceinline__ float3 single_total(const DevScene& S, const KParams& kp, const float* dI, float4 a,
+                                               float4 b) {
+  const float3 L = f3(b.y, b.z, b.w);
+  return mul(adjoint_read_f(dI, S.W, S.H, a.w, b.x, L, nullptr, kp.filter), L);
+}
+
 // ======================================================================= LRB-3-pass
 // Pass 2 (accumulate delta_total, Eq. 14) and pass 3 (backpropagate, Eq. 15-17) per path,
 // run as a per-lane state machine: every iteration of the step loop performs one vertex
@@ -1268,18 +1332,23 @@ __global__ void __launch_bounds__(256) k_primal_batch(BatchArgs ba) {
 // BATCH: per-lane item (BatchDispenser), global gradient atomics, per-item attached flag;
 // S0, kp0, dI0 and g0 are not used.
 // MODE 0: passes 2 and 3 fused per lane.  MODE 1: pass 2 only, storing delta_total and the
-// validity mask of path p in xrec[p] (rgb, bits 0-31) and xhi[p] (bits 32-63).  MODE 2:
-// pass 3 only, starting from that state (paths without a valid connection are skipped).
-// MK (MODE 1): the primal stored each path's validity mask in xrec/xhi, so pass 2 takes
-// connection validity from it, traces no visibility rays, stops after the last valid
-// connection and skips paths without one.
+// validity mask of a path in its state (PathState).  MODE 2: pass 3 only, starting from that
+// state (paths without a valid connection are skipped).
+// MK (MODE 1): the primal stored each path's validity mask, so pass 2 takes connection validity
+// from it, traces no visibility rays, stops after the last valid connection and skips paths
+// without one, and paths with one: k_lrb3_single forms their delta_total (a batch does it here).
 // LOCAL: the calling block alone works on the path range (a span of a batch item).
-// With a path list (kp.list, masks known): MODE 1 (MK) and MODE 2 visit only the listed
-// paths, the ones with a valid connection, so no lane draws a path it has nothing to do for.
+// With a path list (kp.list, masks known): MODE 1 (MK) visits only the listed paths with
+// several connections and MODE 2 the listed ones, so no lane draws a path it has nothing to do
+// for.
+// Known hits (kp.hits, from the primal's records): both passes intersect the recorded primitive
+// at a path's first vertices, which gives the search's hit bit for bit, and search the scene
+// only beyond them.  Box, 2^22 paths, depth 16 (11 bits a hit, 14 of
+// them in pass 3): pass 2 4.22 -> 1.24 ms, pass 3 7.62 -> 4.55 ms; caustic, 2^24 paths (16 bits):
+// pass 3 3.7 -> 2.65 ms, pass 2 0.27 -> 0.05 ms.
 template <bool ATT, bool ST, bool CH, bool BATCH, int MODE = 0, bool MK = false, bool LOCAL = false>
 __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0, const float* __restrict__ dI0,
-                                          const GradPtrs& g0, const BatchArgs& ba, float4* xrec = nullptr,
-                                          uint32_t* xhi = nullptr) {
+                                          const GradPtrs& g0, const BatchArgs& ba, const PathState& st0 = {}) {
   extern __shared__ float sgrad[];
   GradPtrs gs = g0;
   if (!BATCH) {
@@ -1294,10 +1363,12 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   Dispenser disp;
   BatchDispenser bdisp;
   // the path list applies to pass 2 with known masks and to pass 3
-  const uint32_t* list = (!BATCH && !LOCAL && (MODE == 2 || (MODE == 1 && MK))) ? kp0.list : nullptr;
+  const uint32_t* list = BATCH || LOCAL ? nullptr : MODE == 2 ? kp0.list : (MODE == 1 && MK) ? kp0.multi : nullptr;
   if (BATCH) bdisp.init();
   else if (LOCAL) disp.init_local(kp0.n_paths);
-  else if (list) disp.init_dynamic(min((int64_t)*kp0.list_n, kp0.n_paths), kp0.ticket + (MODE == 1 ? 0 : 1));
+  else if (list)
+    disp.init_dynamic(min((int64_t) * (MODE == 1 ? kp0.multi_n : kp0.list_n), kp0.n_paths),
+                      kp0.ticket + (MODE == 1 ? 0 : 1));
   else disp.init(kp0.n_paths);
   int jb = 0;
   // FLUSH: the lane's path is done except the reverse sweep through the specular chain that
@@ -1320,6 +1391,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   // a chain's reverse sweep along those of the walk it ends
   constexpr bool LOG = CH || MODE == 0;
   HitLog log;
+  constexpr bool HITS = MODE == 2 || (MODE == 1 && MK);
+  HitWords<MODE == 2 ? 5 : 8> hw;  // the path's recorded primitives, valid below vertex hcap
+  int hcap = 0;
   TravState ts;  // the lane's ray in flight (see TravState)
   LocalStack stk;
   bool inflight = false;
@@ -1327,24 +1401,24 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   auto start = [&](int64_t got) {
     const DevScene& S = BATCH ? ba.jobs[jb].S : S0;
     const KParams& kp = BATCH ? ba.jobs[jb].kp : kp0;
-    float4* xr = xrec;
-    uint32_t* xh = xhi;
-    if (BATCH && MODE != 0) {
-      xr = (float4*)ba.jobs[jb].state;
-      xh = (uint32_t*)((char*)ba.jobs[jb].state + lrb3_state_split(kp.n_paths));
-    }
+    const PathState ps = BATCH && MODE != 0 ? path_state(ba.jobs[jb].state, kp.n_paths) : st0;
     if (got >= 0 && list) got = (int64_t)list[got];
     if (got < 0) {
       more = false;
     } else if (MODE == 2) {
-      const float4 a = xr[got];
-      const uint64_t vm = (uint64_t)__float_as_uint(a.w) | ((uint64_t)xh[got] << 32);
+      const uint64_t vm = (uint64_t)ps.mlo[got] | ((uint64_t)ps.mhi[got] << 32);
       if (vm && (!kp.mask || kp.mask[got])) {
         p = got;
+        const float4 a = ps.a[ps.step * p], b = ps.b[ps.step * p];
+        if constexpr (MODE == 2) {
+          hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
+          hw.w[3] = __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x);
+          hcap = kp.hits.bits == 0 ? 0 : (vm & (vm - 1)) == 0ull ? kp.hits.cap1 : kp.hits.cap3;
+        }
         if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
         float3 x0;
         walk_start(S, kp.seed, (uint64_t)(kp.path_offset + p), Le, w, x0);
-        rem = f3(a.x, a.y, a.z);
+        rem = f3(b.y, b.z, b.w);
         valid = vm;
         pend_init(pv, -1, -1, 0.0f, 0.0f, x0, S.ln);
         chain.ka = -1;
@@ -1354,15 +1428,30 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         phase = PASS3;
       }
     } else if (!kp.mask || kp.mask[got]) {
-      if (MK) known = (uint64_t)__float_as_uint(xr[got].w) | ((uint64_t)xh[got] << 32);
+      if (MK) known = (uint64_t)ps.mlo[got] | ((uint64_t)ps.mhi[got] << 32);
       if (MK && !known) {  // no valid connection: delta_total = 0, the stored state stands
         if (kp.dbg) ((float4*)kp.dbg)[got] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         return;
       }
-      // one valid connection: k_lrb3_single has formed its delta_total without a replay
-      if (MODE == 1 && MK && !BATCH && kp.conn1 && (known & (known - 1)) == 0ull) return;
-      p = got;
       if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
+      if constexpr (MODE == 1 && MK) {
+        const bool one = (known & (known - 1)) == 0ull;
+        // one valid connection: k_lrb3_single has formed its delta_total without a replay
+        if (!BATCH && one) return;
+        const float4 a = ps.a[ps.step * got], b = ps.b[ps.step * got];
+        if (one) {
+          const float3 d = single_total(S, kp, ba.jobs[jb].dI, a, b);
+          ps.b[ps.step * got] = make_float4(b.x, d.x, d.y, d.z);
+          gLe = gLe + f3(d.x / Le.x, d.y / Le.y, d.z / Le.z);
+          if (kp.dbg) ((float4*)kp.dbg)[got] = make_float4(d.x, d.y, d.z, 1.0f);
+          return;
+        }
+        hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
+        hw.w[3] = __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = __float_as_uint(b.y);
+        hw.w[6] = __float_as_uint(b.z); hw.w[7] = __float_as_uint(b.w);
+        hcap = kp.hits.bits == 0 ? 0 : kp.hits.cap;
+      }
+      p = got;
       float3 x0;
       walk_start(S, kp.seed, (uint64_t)(kp.path_offset + p), Le, w, x0);
       dtot = f3(0, 0, 0);
@@ -1411,21 +1500,28 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     const GradPtrs& g = BATCH ? ba.jobs[jb].g : gs;
     const bool att = ATT && (!BATCH || ba.jobs[jb].att);
     // per-path state of the two-kernel form (the lane's item's, in a batch)
-    float4* xr = xrec;
-    uint32_t* xh = xhi;
-    if (BATCH && MODE != 0) {
-      xr = (float4*)ba.jobs[jb].state;
-      xh = (uint32_t*)((char*)ba.jobs[jb].state + lrb3_state_split(kp.n_paths));
-    }
+    const PathState ps = BATCH && MODE != 0 ? path_state(ba.jobs[jb].state, kp.n_paths) : st0;
     if (!__any_sync(0xffffffffu, phase != IDLE || more)) break;
     // pass 2 with known masks also stops after the path's last valid connection
     const int kmax = phase == PASS2 && !MK ? kp.max_depth : last + 1;
-    const bool trav = (phase == PASS2 || phase == PASS3) && k < kmax && !w.dead;
+    bool trav = (phase == PASS2 || phase == PASS3) && k < kmax && !w.dead;
     HitRec h;
     h.prim = -1;
     bool pending = false;  // the ray has visits left: the lane resumes it in the next step
+    if constexpr (HITS) {
+      // few lanes are beyond their recorded hits at a time: they wait until kSearchBatch lanes of
+      // the warp are (or no other lane has work) and search together
+      const bool known = trav && k < hcap, search = trav && !known;
+      const unsigned sq = __ballot_sync(0xffffffffu, search), kq = __ballot_sync(0xffffffffu, known);
+      if (search && kq != 0u && __popc(sq) < kSearchBatch) {
+        pending = true;
+        trav = false;
+      }
+    }
     if (MODE == 0 && trav && phase == PASS3) {
       h = hit_known(S, w.org, w.dir, log(k));
+    } else if (HITS && trav && k < hcap) {
+      h = hit_known(S, w.org, w.dir, hw.get(kp.hits, k, S.n_prims));
     } else if constexpr (CH) {
       // the specular-chain variants keep whole traversals: the resumable state would
       // push them past the register budget that their chain transport needs
@@ -1484,8 +1580,13 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(dtot.x, dtot.y, dtot.z, (float)nconn);
         gLe = gLe + f3(dtot.x / Le.x, dtot.y / Le.y, dtot.z / Le.z);  // emitted factor, weight delta_total
         if (MODE == 1) {
-          xr[p] = make_float4(dtot.x, dtot.y, dtot.z, __uint_as_float((uint32_t)valid));
-          xh[p] = (uint32_t)(valid >> 32);
+          if constexpr (MODE == 1) {
+            ps.b[ps.step * p] = make_float4(MK ? __uint_as_float(hw.w[4]) : 0.0f, dtot.x, dtot.y, dtot.z);
+            if (!MK) {
+              ps.mlo[p] = (uint32_t)valid;
+              ps.mhi[p] = (uint32_t)(valid >> 32);
+            }
+          }
           phase = IDLE;
         } else if (valid) {
           float3 x0;
@@ -1572,30 +1673,41 @@ __global__ void __launch_bounds__(128, 4) k_lrb3(DevScene S, KParams kp, const f
 // caustic backward from 8.8 to 7.4 ms, while the lean pass 3 (no chains) was fastest at 4.
 template <bool ST, bool MK>
 __global__ void __launch_bounds__(128, 6) k_lrb3_p2(DevScene S, KParams kp, const float* __restrict__ dI, GradPtrs g0,
-                                                 float4* xrec, uint32_t* xhi) {
-  lrb3_body<false, ST, false, false, 1, MK>(S, kp, dI, g0, BatchArgs{}, xrec, xhi);
+                                                 PathState ps) {
+  lrb3_body<false, ST, false, false, 1, MK>(S, kp, dI, g0, BatchArgs{}, ps);
 }
 // Pass 2 of the paths with exactly one valid connection (known masks, the primal's record of
-// each path's first valid connection): delta_total = Lbar (.) L of that connection (Eq. 14)
-// from its recorded film position and contribution, the values a replay computes, one thread
-// per listed path; k_lrb3_p2 leaves these paths out.  On the caustic workload they are 98 %
-// of the paths with a connection.
+// the connection): delta_total = Lbar (.) L of that connection (Eq. 14) from its recorded film
+// position and contribution, the values a replay computes, one thread per listed path.  The
+// listed paths with several connections are collected for k_lrb3_p2.  On the caustic workload
+// 98 % of the paths with a connection have one.
 __global__ void __launch_bounds__(256) k_lrb3_single(DevScene S, KParams kp, const float* __restrict__ dI,
-                                                    GradPtrs g, float4* xrec, const uint32_t* xhi) {
+                                                    GradPtrs g, PathState ps) {
   const int64_t n = kp.list ? min((int64_t)*kp.list_n, kp.n_paths) : kp.n_paths;
   const float3 Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
   float3 gLe = f3(0, 0, 0);
   unsigned long long ones = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = kp.list ? (int64_t)kp.list[i] : i;
-    if (kp.mask && !kp.mask[p]) continue;
-    const float4 r = xrec[p];
-    const uint64_t known = (uint64_t)__float_as_uint(r.w) | ((uint64_t)xhi[p] << 32);
-    if (known == 0ull || (known & (known - 1)) != 0ull) continue;
-    const float4 a = kp.conn1[p];
-    const float3 L = f3(a.z, a.w, kp.conn1z[p]);
-    const float3 d = mul(adjoint_read_f(dI, S.W, S.H, a.x, a.y, L, nullptr, kp.filter), L);
-    xrec[p] = make_float4(d.x, d.y, d.z, r.w);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
+    const int64_t i = base + threadIdx.x;
+    const int64_t p = i < n ? (kp.list ? (int64_t)kp.list[i] : i) : -1;
+    const bool in = p >= 0 && (!kp.mask || kp.mask[p]);
+    const uint64_t known = in ? (uint64_t)ps.mlo[p] | ((uint64_t)ps.mhi[p] << 32) : 0ull;
+    const bool several = (known & (known - 1)) != 0ull;
+    if (kp.multi) {
+      const unsigned b = __ballot_sync(0xffffffffu, several);
+      if (b) {
+        const int lane = threadIdx.x & 31, leader = __ffs(b) - 1;
+        unsigned long long at = 0;
+        if (lane == leader) at = atomicAdd(kp.multi_n, (unsigned long long)__popc(b));
+        at = __shfl_sync(0xffffffffu, at, leader);
+        if (several) kp.multi[at + __popc(b & ((1u << lane) - 1u))] = (uint32_t)p;
+      }
+    }
+    if (known == 0ull || several) continue;
+    const float4 a = ps.a[ps.step * p], r = ps.b[ps.step * p];
+    const float3 d = single_total(S, kp, dI, a, r);
+    ps.b[ps.step * p] = make_float4(r.x, d.x, d.y, d.z);
     gLe = gLe + f3(d.x / Le.x, d.y / Le.y, d.z / Le.z);  // emitted factor, weight delta_total
     ++ones;
     if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(d.x, d.y, d.z, 1.0f);
@@ -1611,9 +1723,8 @@ __global__ void __launch_bounds__(256) k_lrb3_single(DevScene S, KParams kp, con
 // ... then pass 3 (albedo and height gradients) from that state.
 template <bool ATT, bool ST, bool CH>
 __global__ void __launch_bounds__(128, CH ? 8 : 4) k_lrb3_p3(DevScene S, KParams kp, const float* __restrict__ dI, GradPtrs g0,
-                                                 const float4* xrec, const uint32_t* xhi) {
-  lrb3_body<ATT, ST, CH, false, 2>(S, kp, dI, g0, BatchArgs{}, const_cast<float4*>(xrec),
-                                   const_cast<uint32_t*>(xhi));
+                                                 PathState ps) {
+  lrb3_body<ATT, ST, CH, false, 2>(S, kp, dI, g0, BatchArgs{}, ps);
 }
 
 // Batched two-kernel form: pass 2 over every item, then pass 3 per kernel group.
@@ -1647,13 +1758,16 @@ __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restric
     kp.n_paths = span.end - span.start;
     if (kp.mask) kp.mask += span.start;
     if (kp.dbg) kp.dbg += 4 * span.start;
-    float4* xr = (float4*)J.state + span.start;
-    uint32_t* xh = (uint32_t*)((char*)J.state + lrb3_state_split(J.kp.n_paths)) + span.start;
+    PathState ps = path_state(J.state, J.kp.n_paths);
+    ps.a += ps.step * span.start;
+    ps.b += ps.step * span.start;
+    ps.mlo += span.start;
+    ps.mhi += span.start;
     GradPtrs g = J.g;
     g.d_Le = nullptr;  // pass 2 added the emitted-radiance gradient
     const bool att = ATT && J.att;
-    if (att) lrb3_body<ATT, false, CH, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, xr, xh);
-    else lrb3_body<false, false, false, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, xr, xh);
+    if (att) lrb3_body<ATT, false, CH, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
+    else lrb3_body<false, false, false, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
   }
 }
 
@@ -1824,8 +1938,7 @@ __global__ void __launch_bounds__(256) k_reslrb_batch(BatchArgs ba) {
 __global__ void __launch_bounds__(128) k_lrb2_reduce(DevScene S, KParams kp, const float* __restrict__ dI,
                                                      void* buf, float* d_Le) {
   const Lrb2Layout lay = lrb2_layout(kp.n_paths, kp.max_depth);
-  float4* xrec = (float4*)buf;
-  uint32_t* xhi = (uint32_t*)((char*)buf + lrb3_state_split(kp.n_paths));
+  const PathState ps = lrb2_path_state(buf, kp.n_paths, kp.max_depth);
   const int* cnt = (const int*)((const char*)buf + lay.counts);
   const float4* r4 = (const float4*)((const char*)buf + lay.rec4);
   const float* rz = (const float*)((const char*)buf + lay.recz);
@@ -1847,8 +1960,10 @@ __global__ void __launch_bounds__(128) k_lrb2_reduce(DevScene S, KParams kp, con
       valid |= 1ull << k;
       ++nconn;
     }
-    xrec[p] = make_float4(dtot.x, dtot.y, dtot.z, __uint_as_float((uint32_t)valid));
-    xhi[p] = (uint32_t)(valid >> 32);
+    float4* rec = ps.b + ps.step * p;
+    rec->y = dtot.x; rec->z = dtot.y; rec->w = dtot.z;
+    ps.mlo[p] = (uint32_t)valid;
+    ps.mhi[p] = (uint32_t)(valid >> 32);
     gLe = gLe + f3(dtot.x / Le.x, dtot.y / Le.y, dtot.z / Le.z);  // emitted factor, weight delta_total
     if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(dtot.x, dtot.y, dtot.z, (float)nconn);
   }
@@ -2713,6 +2828,7 @@ cudaError_t launch_primal(const DevScene& S, const KParams& kp, int est, float* 
     case 0:
       if (kp.census) launch_paths(k_primal_census, L, kp.n_paths, 0, st, S, kp, image, aux);
       else if (S.atomics == 2) launch_paths(k_primal_agg, L, kp.n_paths, 0, st, S, kp, image, aux);
+      else if (kp.vstate) launch_paths(k_primal<0, true>, L, kp.n_paths, 0, st, S, kp, image, aux);
       else launch_paths(k_primal<0>, L, kp.n_paths, 0, st, S, kp, image, aux);
       break;
     case 1:
@@ -2729,29 +2845,27 @@ cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool cha
                         const GradPtrs& g, void* state, bool mask_ready, const LaunchCfg& L, cudaStream_t st) {
   const size_t smem = kp.priv_n > 0 ? sizeof(float) * (size_t)kp.priv_n : 0;
   if (state) {
-    float4* xrec = (float4*)state;
-    uint32_t* xhi = (uint32_t*)((char*)state + lrb3_state_split(kp.n_paths));
+    const PathState ps = path_state(state, kp.n_paths);
     KParams k2 = kp;
     k2.priv_n = 0;  // pass 2 writes no albedo or height gradients
     GradPtrs g3 = g;
     g3.d_Le = nullptr;  // pass 3 writes no emitted-radiance gradient
-    if (mask_ready && kp.conn1)
-      k_lrb3_single<<<L.sms * 4, 256, 0, st>>>(S, k2, dI, g, xrec, xhi);
+    if (mask_ready) k_lrb3_single<<<L.sms * 4, 256, 0, st>>>(S, k2, dI, g, ps);
     if (kp.census) {
-      if (mask_ready) launch_paths(k_lrb3_p2<true, true>, L, kp.n_paths, 0, st, S, k2, dI, g, xrec, xhi);
-      else launch_paths(k_lrb3_p2<true, false>, L, kp.n_paths, 0, st, S, k2, dI, g, xrec, xhi);
+      if (mask_ready) launch_paths(k_lrb3_p2<true, true>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
+      else launch_paths(k_lrb3_p2<true, false>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
     } else {
-      if (mask_ready) launch_paths(k_lrb3_p2<false, true>, L, kp.n_paths, 0, st, S, k2, dI, g, xrec, xhi);
-      else launch_paths(k_lrb3_p2<false, false>, L, kp.n_paths, 0, st, S, k2, dI, g, xrec, xhi);
+      if (mask_ready) launch_paths(k_lrb3_p2<false, true>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
+      else launch_paths(k_lrb3_p2<false, false>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
     }
     if (kp.census) {
-      if (att && chains) launch_paths(k_lrb3_p3<true, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-      else if (att) launch_paths(k_lrb3_p3<true, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-      else launch_paths(k_lrb3_p3<false, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
+      if (att && chains) launch_paths(k_lrb3_p3<true, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else if (att) launch_paths(k_lrb3_p3<true, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else launch_paths(k_lrb3_p3<false, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
     } else {
-      if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-      else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-      else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
+      if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
     }
     return cudaGetLastError();
   }
@@ -2788,14 +2902,13 @@ cudaError_t launch_naive(const DevScene& S, const KParams& kp, bool att, bool ch
 cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI, void* buf,
                         const GradPtrs& g, const LaunchCfg& L, cudaStream_t st) {
   launch_paths(k_lrb2_reduce, L, kp.n_paths, 0, st, S, kp, dI, buf, g.d_Le);
-  float4* xrec = (float4*)buf;
-  uint32_t* xhi = (uint32_t*)((char*)buf + lrb3_state_split(kp.n_paths));
+  const PathState ps = lrb2_path_state(buf, kp.n_paths, kp.max_depth);
   const size_t smem = kp.priv_n > 0 ? sizeof(float) * (size_t)kp.priv_n : 0;
   GradPtrs g3 = g;
   g3.d_Le = nullptr;  // added by the reduction
-  if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-  else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
-  else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, xrec, xhi);
+  if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+  else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+  else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
   return cudaGetLastError();
 }
 

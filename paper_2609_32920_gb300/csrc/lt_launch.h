@@ -7,6 +7,13 @@ namespace lt {
 
 struct DevScene;
 
+// Primitives of a path's first vertices as kept in its per-path record: `bits` each (enough for
+// the scene's primitives), at most `cap` of them for pass 2 (256 bits) and `cap3` for pass 3
+// (160 bits, or `cap1` in 96 bits for a path with one valid connection); see lrb3_state_bytes.
+struct HitBits {
+  int bits, cap, cap3, cap1;
+};
+
 // Per-call kernel parameters (by value).
 struct KParams {
   uint64_t seed;
@@ -36,9 +43,9 @@ struct KParams {
   unsigned long long* list_n;  // length of `list`
   unsigned long long* ticket;  // zeroed counters of entries taken: [0] pass 2, [1] pass 3 (plain
                                // primal with the LRB-3 state: [0] its 32-path chunks)
-  float4* conn1;               // per path: film position and contribution (u_x, u_y, L.r, L.g) of
-  float* conn1z;               // its first valid connection, and L.b (plain primal: writes; LRB-3
-                               // pass 2 with known masks: reads for paths with one connection)
+  uint32_t* multi;             // LRB-3 backward with a list: its paths with several connections
+  unsigned long long* multi_n; // (k_lrb3_single appends, pass 2 visits), and their number
+  HitBits hits;                // primitives kept in the per-path records (bits 0: none)
   int jac_noise;               // paper-literal transport: Jacobian noise at diffuse vertices
   uint64_t noise_seed;         // its Philox key
   float det_eps;               // its determinant guard
@@ -119,47 +126,74 @@ namespace w4 { LT_KERNEL_LAUNCHERS }
 namespace w8 { LT_KERNEL_LAUNCHERS }
 LT_KERNEL_LAUNCHERS
 
-// `state` of launch_lrb3 (or null: fused kernel): per-path state of the two-kernel form,
-// layout float4[n_paths] then, at byte lrb3_state_split(n_paths), uint32[n_paths] (together
-// lrb3_state_core bytes); then the list of the paths that have a valid connection (uint32
-// indices relative to the call, at lrb3_state_list) and its length (uint64, at
-// lrb3_state_count), written by a plain primal so that passes 2 and 3 visit only those;
-// then each path's first valid connection, float4 (u_x, u_y, L.r, L.g) at lrb3_state_conn4
-// and float L.b at lrb3_state_connz, written by the plain primal; then the order in which the
-// plain primal takes the paths (uint32[n_paths] at lrb3_state_order) and the counting sort's
-// work area that builds it (kSortBins x kSortBlocks counts, then kSortBins bin starts).
+// `state` of launch_lrb3 (or null: fused kernel): per-path state of the two-kernel form.
+//  - a record of 32 B per path (at 0), eight words: words 5-7 are delta_total once pass 2 has
+//    formed it.  The plain primal keeps there, for a path with a valid connection, the
+//    primitives of its first vertices (HitBits, packed from bit 0 upwards), so that the passes
+//    intersect the known primitive instead of searching the scene: a path with several valid
+//    connections has words 0-7 for them until pass 2 writes delta_total and words 0-4 then; a
+//    path with one valid connection has words 0-2, and words 3-7 hold the film position and the
+//    contribution (u_x, u_y, L.rgb) of that connection.  One aligned sector per path, because
+//    the passes visit the paths in the order of the list and gather it.
+//  - validity bits 0-31 (at lrb3_state_mlo) and 32-63 (at lrb3_state_mhi), uint32 each;
+//  - the list of the paths that have a valid connection (uint32 indices relative to the call, at
+//    lrb3_state_list), written by the plain primal so that passes 2 and 3 visit only those, and
+//    256 B of counters at lrb3_state_count: its length, the passes' counters of entries taken
+//    (two), the number of listed paths with several connections (uint64 each);
+//  - the order in which the plain primal takes the paths (uint32[n_paths] at lrb3_state_order;
+//    the backward reuses the array for the listed paths with several connections) and the
+//    counting sort's work area that builds it (kSortBins x kSortBlocks counts, then kSortBins
+//    bin starts).
+// In all 48 B per path, flat in depth.
 constexpr int kSortBins = 4096;   // 64 x 64 cells of the first direction
 constexpr int kSortBlocks = 256;  // blocks of the sort, each over a contiguous range of paths
 __host__ __device__ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-__host__ __device__ inline size_t lrb3_state_split(int64_t n) { return align256((size_t)n * 16); }
-__host__ __device__ inline size_t lrb3_state_core(int64_t n) { return lrb3_state_split(n) + align256((size_t)n * 4); }
+__host__ __device__ inline size_t lrb3_state_mlo(int64_t n) { return align256((size_t)n * 32); }
+__host__ __device__ inline size_t lrb3_state_mhi(int64_t n) { return lrb3_state_mlo(n) + align256((size_t)n * 4); }
+__host__ __device__ inline size_t lrb3_state_core(int64_t n) { return lrb3_state_mhi(n) + align256((size_t)n * 4); }
 __host__ __device__ inline size_t lrb3_state_list(int64_t n) { return lrb3_state_core(n); }
 __host__ __device__ inline size_t lrb3_state_count(int64_t n) { return lrb3_state_list(n) + align256((size_t)n * 4); }
-__host__ __device__ inline size_t lrb3_state_conn4(int64_t n) { return lrb3_state_count(n) + 256; }
-__host__ __device__ inline size_t lrb3_state_connz(int64_t n) { return lrb3_state_conn4(n) + align256((size_t)n * 16); }
-__host__ __device__ inline size_t lrb3_state_order(int64_t n) { return lrb3_state_connz(n) + align256((size_t)n * 4); }
+__host__ __device__ inline size_t lrb3_state_order(int64_t n) { return lrb3_state_count(n) + 256; }
 __host__ __device__ inline size_t lrb3_state_sort(int64_t n) { return lrb3_state_order(n) + align256((size_t)n * 4); }
 __host__ __device__ inline size_t lrb3_state_bytes(int64_t n) {
   return lrb3_state_sort(n) + align256(sizeof(unsigned) * (size_t)kSortBins * (kSortBlocks + 1));
 }
-// After the list's length (uint64) at lrb3_state_count: the two passes' counters of list
-// entries taken (uint64 each).
+// The per-path arrays of a state (or of the buffered two-pass buffer) of n paths: words 0-3 and
+// 4-7 of the record of path p are at a[step * p] and b[step * p].
+struct PathState {
+  float4 *a, *b;
+  uint32_t *mlo, *mhi;
+  int step;
+};
+__host__ __device__ inline PathState path_state(void* base, int64_t n) {
+  char* c = (char*)base;
+  return PathState{(float4*)c, (float4*)c + 1, (uint32_t*)(c + lrb3_state_mlo(n)), (uint32_t*)(c + lrb3_state_mhi(n)), 2};
+}
 // The path list is used for calls of at most this many paths (uint32 indices).
 constexpr int64_t kListMaxPaths = 0xffffffffll;
 
-// Buffer of the buffered two-pass estimator (lrb_2pass): the LRB-3 per-path state, then
-// per path its traced vertex count (int), then per vertex [depth][path] the splat record
-// (u_x, u_y, L.r, L.g) (float4; u_x < 0 = no valid connection) and L.b (float).
+// Buffer of the buffered two-pass estimator (lrb_2pass): per path words 4-7 of an LRB-3 record
+// (16 B), validity bits 32-63 and its traced vertex count (int), then per vertex [depth][path]
+// the splat record (u_x, u_y, L.r, L.g) (float4; u_x < 0 = no valid connection) and L.b
+// (float), then per path words 0-3 of the record and validity bits 0-31.
 struct Lrb2Layout {
-  size_t counts, rec4, recz, total;
+  size_t mhi, counts, rec4, recz, rec0, mlo, total;
 };
 __host__ __device__ inline Lrb2Layout lrb2_layout(int64_t n, int d) {
   Lrb2Layout L;
-  L.counts = lrb3_state_core(n);
+  L.mhi = align256((size_t)n * 16);
+  L.counts = L.mhi + align256((size_t)n * 4);
   L.rec4 = L.counts + align256((size_t)n * 4);
   L.recz = L.rec4 + align256((size_t)n * (size_t)d * 16);
-  L.total = L.recz + align256((size_t)n * (size_t)d * 4);
+  L.rec0 = L.recz + align256((size_t)n * (size_t)d * 4);
+  L.mlo = L.rec0 + align256((size_t)n * 16);
+  L.total = L.mlo + align256((size_t)n * 4);
   return L;
+}
+__host__ __device__ inline PathState lrb2_path_state(void* buf, int64_t n, int d) {
+  const Lrb2Layout L = lrb2_layout(n, d);
+  char* c = (char*)buf;
+  return PathState{(float4*)(c + L.rec0), (float4*)c, (uint32_t*)(c + L.mlo), (uint32_t*)(c + L.mhi), 1};
 }
 size_t mlp_grad_smem_bytes();
 cudaError_t launch_mlp_grad(const float* P, const float* X, const float* T, int64_t n, float inv_batch, float* g,
