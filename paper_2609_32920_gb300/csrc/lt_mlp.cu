@@ -2,6 +2,7 @@
 // tensor cores: forward and backward GEMM tiles on mma.sync.m16n8k16 (BF16 operands, FP32
 // accumulation), per-block gradient accumulation in shared memory, Adam update, and the
 // feature/target standardisation statistics.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "lt_launch.h"
@@ -249,33 +250,70 @@ __global__ void k_mlp_adam(float* __restrict__ P, float* __restrict__ Mm, float*
   P[i] -= lr * mh / (sqrtf(vh) + eps);
 }
 
-// Mean and standard deviation of every feature and of the target, written into the
-// parameter block (one block, FP64 sums; used once per training set).
+// Mean and standard deviation of every feature and of the target, written into the parameter
+// block (FP64 sums).  One cluster of kMomBlocks blocks: FP64 arithmetic bounds it (two adds per
+// value at two a clock and SM), so the rows are split over the cluster's SMs and the blocks' sums
+// meet in the first block's shared memory.  Sixteen SMs took 2^17 rows from 2445 us (one block) to
+// 154 us; a grid of independent blocks would need a workspace that the call does not have.
+constexpr int kMomBlocks = 16;
 __global__ void __launch_bounds__(1024) k_mlp_moments(const float* __restrict__ X, const float* __restrict__ T,
                                                       int64_t n, float* __restrict__ P) {
-  __shared__ double sh[17][2];
-  if (threadIdx.x < 34) (&sh[0][0])[threadIdx.x] = 0.0;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double sh[34];
+  __shared__ double all[kMomBlocks][34];  // read in block 0
+  if (threadIdx.x < 34) sh[threadIdx.x] = 0.0;
   __syncthreads();
-  double loc[17][2] = {};
-  for (int64_t s = threadIdx.x; s < n; s += blockDim.x) {
-    for (int i = 0; i < 16; ++i) {
-      const double v = X[s * 16 + i];
-      loc[i][0] += v;
-      loc[i][1] += v * v;
+  // thread = (row, quarter of its features): 16 B loads, and the targets with the first quarter
+  const int q = threadIdx.x & 3;
+  double a[5] = {}, b[5] = {};
+  const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 4);
+  for (int64_t s = (int64_t)blockIdx.x * (blockDim.x / 4) + (threadIdx.x >> 2); s < n; s += stride) {
+    const float* x = X + s * 16 + 4 * q;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double v = x[i];
+      a[i] += v;
+      b[i] += v * v;
     }
-    const double t = T[s];
-    loc[16][0] += t;
-    loc[16][1] += t * t;
+    if (q == 0) {
+      const double t = T[s];
+      a[4] += t;
+      b[4] += t * t;
+    }
   }
-  for (int i = 0; i < 17; ++i) {
-    atomicAdd(&sh[i][0], loc[i][0]);
-    atomicAdd(&sh[i][1], loc[i][1]);
+  // over the rows of the warp, then of the block
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+      a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
+      b[i] += __shfl_xor_sync(0xffffffffu, b[i], o);
+    }
+  if ((threadIdx.x & 31) < 4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      atomicAdd(&sh[2 * (4 * q + i)], a[i]);
+      atomicAdd(&sh[2 * (4 * q + i) + 1], b[i]);
+    }
+    if (q == 0) {
+      atomicAdd(&sh[32], a[4]);
+      atomicAdd(&sh[33], b[4]);
+    }
   }
   __syncthreads();
+  double* dst = cluster.map_shared_rank(&all[0][0], 0);
+  if (threadIdx.x < 34) dst[cluster.block_rank() * 34 + threadIdx.x] = sh[threadIdx.x];
+  cluster.sync();
   const int i = threadIdx.x;
-  if (i < 17) {
-    const double mean = sh[i][0] / (double)n;
-    const double var = sh[i][1] / (double)n - mean * mean;
+  if (cluster.block_rank() == 0 && i < 17) {
+    double s0 = 0.0, s1 = 0.0;
+    for (int k = 0; k < (int)cluster.num_blocks(); ++k) {
+      s0 += all[k][2 * i];
+      s1 += all[k][2 * i + 1];
+    }
+    const double mean = s0 / (double)n;
+    const double var = s1 / (double)n - mean * mean;
     const double sd = sqrt(var > 1e-12 ? var : 1e-12);
     if (i < 16) {
       P[kOffMean + i] = (float)mean;
@@ -332,8 +370,31 @@ cudaError_t launch_mlp_adam(float* P, float* M, float* V, const float* g, int st
 }
 
 cudaError_t launch_mlp_moments(const float* X, const float* T, int64_t n, float* P, cudaStream_t st) {
-  k_mlp_moments<<<1, 1024, 0, st>>>(X, T, n, P);
-  return cudaGetLastError();
+  // fewer rows than a cluster of blocks holds in a few passes: a smaller cluster, down to one block
+  int blocks = kMomBlocks;
+  while (blocks > 1 && n < (int64_t)blocks * 256) blocks /= 2;
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_moments, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(1024);
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = blocks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  // a device that cannot hold that cluster takes a smaller one
+  for (int active = 0; blocks > 1; blocks /= 2) {
+    at.val.clusterDim.x = blocks;
+    cfg.gridDim = dim3(blocks);
+    if (cudaOccupancyMaxActiveClusters(&active, k_mlp_moments, &cfg) == cudaSuccess && active > 0) break;
+    cudaGetLastError();
+  }
+  at.val.clusterDim.x = blocks;
+  cfg.gridDim = dim3(blocks);
+  return cudaLaunchKernelEx(&cfg, k_mlp_moments, X, T, n, P);
 }
 
 cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, float* out, int sms, cudaStream_t st) {
