@@ -158,7 +158,10 @@ typedef struct {
                              in shared memory when the arrays fit in 46 KB, and are added
                              to the caller's arrays once per block; an array that does
                              not fit is added with plain global atomics, and so are the
-                             splats;
+                             splats; pass 3 of lt_backward_lrb3 with lrb3_mask_ready and
+                             of lt_backward_lrb2 instead spreads the albedo gradient over
+                             copies in the state's (buffer's) then unused part and adds
+                             them up, where eight copies or more fit;
                            1 as 0, the per-block arrays up to the device's opt-in shared
                              memory per block (227 KB on GB300; fewer blocks may then be
                              resident per SM);

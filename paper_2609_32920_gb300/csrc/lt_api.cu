@@ -157,6 +157,8 @@ struct lt_scene {
   int device = 0;
   int n_albedo = 0, n_heights = 0, n_tris_h = 0;
   bool has_dielectric = false;
+  int n_mats = 0;
+  int64_t max_texels = 1;  // of a texture
   int sms = 1;
   int smem_optin = 48 * 1024;  // opt-in dynamic shared memory per block
   // device buffers
@@ -359,6 +361,8 @@ KParams kparams(const lt_params* p, const lt_render_opts* o) {
   k.list = nullptr;
   k.list_n = nullptr;
   k.ticket = nullptr;
+  k.rep = nullptr;
+  k.rep_bits = 0;
   k.multi = nullptr;
   k.multi_n = nullptr;
   k.hits = HitBits{0, 0, 0, 0};
@@ -388,6 +392,28 @@ void set_privatization(const lt_scene* s, const lt_grads* g, KParams& kp, int sc
   kp.n_alb = (g && g->d_albedo && s->n_albedo > 0 && s->n_albedo <= budget) ? s->n_albedo : 0;
   kp.n_h = (g && g->d_heights && s->n_heights > 0 && s->n_heights <= budget - kp.n_alb) ? s->n_heights : 0;
   kp.priv_n = kp.n_alb + kp.n_h;
+}
+
+// Copies of the albedo gradient for pass 3 in a work area that the call owns at that point (16-B
+// aligned, `bytes` long): a power of two of entries per material, about one per 256 paths, at
+// least eight per texel of the largest texture.  Where those do not fit: none, and the gradient
+// goes the way set_privatization chose.
+lt_status use_copies(const lt_scene* s, const lt_grads* g, const lt_render_opts* o, void* area, size_t bytes,
+                     KParams& kp, cudaStream_t st) {
+  if (o->scatter != 0 || !g->d_albedo || s->n_albedo < 3) return LT_OK;
+  int least = 8;  // 256 entries (a warp of k_rep_sum) or eight copies of each texel
+  while (least < 40 && (1ll << least) < 8 * s->max_texels) ++least;
+  int most = 0;
+  while (sizeof(float4) * ((size_t)s->n_mats << (most + 1)) <= bytes) ++most;
+  if (most < least || sizeof(float4) * ((size_t)s->n_mats << most) > bytes) return LT_OK;
+  int bits = least;
+  while (bits < most && (256ll << bits) < o->n_paths) ++bits;
+  kp.rep = (float4*)area;
+  kp.rep_bits = bits;
+  kp.priv_n -= kp.n_alb;
+  kp.n_alb = 0;
+  LT_CUDA(cudaMemsetAsync(area, 0, sizeof(float4) * ((size_t)s->n_mats << bits), st));
+  return LT_OK;
 }
 
 lt_status prep_grads(const lt_scene* s, const lt_grads* g, cudaStream_t st, GradPtrs& gp) {
@@ -594,6 +620,10 @@ lt_status lt_scene_create(const lt_scene_desc* d, void* stream, lt_scene** out) 
   s->n_albedo = d->n_albedo;
   s->n_heights = d->n_heights;
   s->has_dielectric = has_diel;
+  s->n_mats = d->n_mats;
+  for (int m = 0; m < d->n_mats; ++m)
+    if (d->mat_type[m] == LT_MAT_DIFFUSE)
+      s->max_texels = std::max(s->max_texels, (int64_t)d->mat_tex_w[m] * d->mat_tex_h[m]);
   s->n_nodes = nn;
   s->n_prims = np;
   auto up = [&](void** dst, const void* src, size_t bytes) -> cudaError_t {
@@ -871,9 +901,14 @@ lt_status lt_backward_lrb3(lt_scene* s, const lt_params* p, const lt_render_opts
     kp.multi_n = kp.list_n + 3;
     kp.multi = (uint32_t*)(base + lrb3_state_order(o->n_paths));
     LT_CUDA(cudaMemsetAsync(kp.ticket, 0, 3 * sizeof(unsigned long long), st));
+    // the sort's work area is free once the primal has run
+    v = use_copies(s, g, o, base + lrb3_state_sort(o->n_paths),
+                   lrb3_state_bytes(o->n_paths) - lrb3_state_sort(o->n_paths), kp, st);
+    if (v != LT_OK) return v;
   }
   cudaError_t e = launch_lrb3(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, gp,
                               o->lrb3_state, o->lrb3_state && o->lrb3_mask_ready, cfg_for(s, o), st);
+  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp.rep, kp.rep_bits, s->n_mats, gp.d_albedo, st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb3: ") + cudaGetErrorString(e));
   return LT_OK;
 }
@@ -911,8 +946,14 @@ lt_status lt_backward_lrb2(lt_scene* s, const lt_params* p, const lt_render_opts
   set_privatization(s, g, kp, o->scatter);
   kp.hits = hit_bits(s);
   kp.hits.cap1 = kp.hits.cap3;  // every record of the buffer has the wide form
-  cudaError_t e = launch_lrb2(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, buf, gp,
-                              cfg_for(s, o), st);
+  const LaunchCfg L = cfg_for(s, o);
+  cudaError_t e = launch_lrb2_reduce(dev_for(s, o), kp, dI, buf, gp, L, st);
+  // the splat records are read: their place serves the copies of the albedo gradient
+  const Lrb2Layout lay = lrb2_layout(o->n_paths, o->max_depth);
+  v = e ? LT_OK : use_copies(s, g, o, (char*)buf + lay.rec4, std::min<size_t>(lay.recz - lay.rec4, 4u << 20), kp, st);
+  if (v != LT_OK) return v;
+  if (!e) e = launch_lrb2(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, buf, gp, L, st);
+  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp.rep, kp.rep_bits, s->n_mats, gp.d_albedo, st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb2: ") + cudaGetErrorString(e));
   return LT_OK;
 }

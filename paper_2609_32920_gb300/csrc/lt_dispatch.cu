@@ -32,6 +32,11 @@ cudaError_t launch_naive(const DevScene& S, const KParams& kp, bool att, bool ch
   return LT_BY_WIDTH(S.width, launch_naive(S, kp, att, chains, dI, ws, g, L, st));
 }
 
+cudaError_t launch_lrb2_reduce(const DevScene& S, const KParams& kp, const float* dI, void* buf, const GradPtrs& g,
+                               const LaunchCfg& L, cudaStream_t st) {
+  return LT_BY_WIDTH(S.width, launch_lrb2_reduce(S, kp, dI, buf, g, L, st));
+}
+
 cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI, void* buf,
                         const GradPtrs& g, const LaunchCfg& L, cudaStream_t st) {
   return LT_BY_WIDTH(S.width, launch_lrb2(S, kp, att, chains, dI, buf, g, L, st));
@@ -40,6 +45,11 @@ cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool cha
 cudaError_t launch_collect(const DevScene& S, const KParams& kp, const float* dI, float tfloor, float* feats,
                            float* targets, int64_t cap, unsigned long long* count, const LaunchCfg& L, cudaStream_t st) {
   return LT_BY_WIDTH(S.width, launch_collect(S, kp, dI, tfloor, feats, targets, cap, count, L, st));
+}
+
+cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,
+                           cudaStream_t st) {
+  return w4::launch_rep_sum(S, rep, rep_bits, n_mats, d_albedo, st);
 }
 
 cudaError_t launch_film_l2(const float* I, const float* T, int64_t n, float* dI, float* loss, int sms,

@@ -330,6 +330,63 @@ __device__ __forceinline__ void scatter_albedo(const DevScene& S, float* g, cons
   }
 }
 
+// The same into copies of the albedo gradient (KParams::rep): every texture has 2^rep_bits
+// entries of 16 B, shared out equally over its texels (rounded up to a power of two), so that a
+// texture of one texel, which gets as many adds as one of 256, is spread as widely: the adds to an
+// address, and with them the rounding of its sum, stay few.  One 16-B reduction per texel.  A
+// shared-memory add of a float is a compare-and-swap loop that the warp waits for, twelve in a row
+// per vertex (335 us for 512 vertices per lane at 8 active lanes of 16 warps per SM); four
+// fire-and-forget vector reductions to copies in L2 take 233 us at the same rate and leave the
+// warp free.  Taps that fall on one texel (edges, one-texel textures) are added first.
+__device__ __forceinline__ int rep_copy_bits(int rep_bits, int texels) {  // log2 of a texel's copies
+  return rep_bits - (texels > 1 ? 32 - __clz(texels - 1) : 0);
+}
+__device__ __forceinline__ void scatter_albedo_rep(float4* rep, int rep_bits, int mat, int4 m, const TexFoot& f,
+                                                   float3 wt, float3 rho) {
+  float3 a = f3(wt.x / rho.x, wt.y / rho.y, wt.z / rho.z);
+  float w[4] = {f.w[0], f.w[1], f.w[2], f.w[3]};
+  if (f.idx[1] == f.idx[0]) { w[0] += w[1]; w[1] = 0.0f; w[2] += w[3]; w[3] = 0.0f; }
+  if (f.idx[2] == f.idx[0]) { w[0] += w[2]; w[2] = 0.0f; w[1] += w[3]; w[3] = 0.0f; }
+  const int cb = rep_copy_bits(rep_bits, m.z * m.w);
+  const unsigned lane = (blockIdx.x * blockDim.x + threadIdx.x) & ((1u << cb) - 1u);
+  float4* base = rep + ((size_t)mat << rep_bits) + lane;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (w[k] == 0.0f) continue;
+    float4* p = base + ((size_t)((unsigned)(f.idx[k] - m.y) / 3u) << cb);
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(a.x * w[k]),
+                 "f"(a.y * w[k]), "f"(a.z * w[k]), "f"(0.0f)
+                 : "memory");
+  }
+}
+// Add the copies up into the caller's array: a warp takes 256 consecutive entries (a texel has
+// eight copies at least), a lane eight of them.
+__global__ void __launch_bounds__(256) k_rep_sum(DevScene S, const float4* __restrict__ rep, int rep_bits, int n_mats,
+                                                 float* d_albedo) {
+  const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  const int mat = (int)(e >> rep_bits);
+  const int4 m = mat < n_mats ? S.mat[mat] : make_int4(-1, 0, 0, 0);
+  const bool in = m.x == MAT_DIFFUSE;
+  const int cb = in ? rep_copy_bits(rep_bits, m.z * m.w) : 8;
+  const int texel = (int)((e & ((1ll << rep_bits) - 1)) >> cb);
+  float3 s = f3(0, 0, 0);
+  if (in && texel < m.z * m.w)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s = s + xyz(rep[e + j]);
+  const int seg = min(32, 1 << (cb - 3));  // lanes with the same texel
+  for (int o = 1; o < seg; o <<= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    s.z += __shfl_xor_sync(0xffffffffu, s.z, o);
+  }
+  if (in && texel < m.z * m.w && (threadIdx.x & (seg - 1)) == 0) {
+    float* d = d_albedo + m.y + 3 * texel;
+    if (s.x != 0.0f) atomicAdd(d, s.x);
+    if (s.y != 0.0f) atomicAdd(d + 1, s.y);
+    if (s.z != 0.0f) atomicAdd(d + 2, s.z);
+  }
+}
+
 // ------------------------------------------------------------ attached local adjoints
 // Attached segment weight (Sec. 3.3 attached samples): g = |n_p.w| |nraw.w| / (|n_p| r^4)
 // for w = x - x_p (the G term times the triangle area); adjoint of log g scaled by lam.
@@ -1356,6 +1413,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     gs.d_albedo = sink.alb;
     gs.d_heights = sink.h;
   }
+  constexpr bool REP = MODE == 2 && !BATCH && !LOCAL;
   float3 Le = BATCH ? f3(0, 0, 0) : f3(kp0.Le[0], kp0.Le[1], kp0.Le[2]);
   float3 gLe = f3(0, 0, 0);
   Census cs = {0, 0, 0};
@@ -1626,7 +1684,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
             rem = rem - P;        // Eq. 16
             if (att) conn_adjoint(S, v.x, v.nraw, hsum(P), q, pv.gx, pv.gn);
           }
-          scatter_albedo(S, g.d_albedo, foot, wsplat + rem, rho);  // + scattering factor rho_k (Eq. 17)
+          // + scattering factor rho_k (Eq. 17)
+          if (REP && kp.rep) scatter_albedo_rep(kp.rep, kp.rep_bits, v.P.mat, v.m, foot, wsplat + rem, rho);
+          else scatter_albedo(S, g.d_albedo, foot, wsplat + rem, rho);
           if (att && CH && !v.attached)
             pv.gx = pv.gx + tex_pos_adjoint(kp.albedo, v.m, v.P, v.b1, v.b2, wsplat + rem, rho);
         }
@@ -2899,9 +2959,14 @@ cudaError_t launch_naive(const DevScene& S, const KParams& kp, bool att, bool ch
   return cudaGetLastError();
 }
 
+cudaError_t launch_lrb2_reduce(const DevScene& S, const KParams& kp, const float* dI, void* buf, const GradPtrs& g,
+                               const LaunchCfg& L, cudaStream_t st) {
+  launch_paths(k_lrb2_reduce, L, kp.n_paths, 0, st, S, kp, dI, buf, g.d_Le);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI, void* buf,
                         const GradPtrs& g, const LaunchCfg& L, cudaStream_t st) {
-  launch_paths(k_lrb2_reduce, L, kp.n_paths, 0, st, S, kp, dI, buf, g.d_Le);
   const PathState ps = lrb2_path_state(buf, kp.n_paths, kp.max_depth);
   const size_t smem = kp.priv_n > 0 ? sizeof(float) * (size_t)kp.priv_n : 0;
   GradPtrs g3 = g;
@@ -3000,6 +3065,13 @@ cudaError_t launch_bidir(const DevScene& S, const KParams& kp, const BidirArgs& 
     if (backward) launch_paths(k_bidir_cam<true>, L, ba.n_cam, smem, st, S, kp, ba, image, dI, g);
     else launch_paths(k_bidir_cam<false>, L, ba.n_cam, smem, st, S, kp, ba, image, dI, g);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,
+                           cudaStream_t st) {
+  const int64_t threads = ((int64_t)n_mats << rep_bits) / 8;
+  k_rep_sum<<<(int)((threads + 255) / 256), 256, 0, st>>>(S, rep, rep_bits, n_mats, d_albedo);
   return cudaGetLastError();
 }
 

@@ -46,6 +46,8 @@ struct KParams {
   uint32_t* multi;             // LRB-3 backward with a list: its paths with several connections
   unsigned long long* multi_n; // (k_lrb3_single appends, pass 2 visits), and their number
   HitBits hits;                // primitives kept in the per-path records (bits 0: none)
+  float4* rep;                 // LRB-3 pass 3: copies of the albedo gradient, [material][2^rep_bits]
+  int rep_bits;                // (see scatter_albedo_rep), or null
   int jac_noise;               // paper-literal transport: Jacobian noise at diffuse vertices
   uint64_t noise_seed;         // its Philox key
   float det_eps;               // its determinant guard
@@ -109,11 +111,16 @@ struct BidirArgs {
                             const void* rec, const GradPtrs& g, const LaunchCfg& L, cudaStream_t st);             \
   cudaError_t launch_naive(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI,           \
                            const void* ws, const GradPtrs& g, const LaunchCfg& L, cudaStream_t st);               \
+  cudaError_t launch_lrb2_reduce(const DevScene& S, const KParams& kp, const float* dI, void* buf,                \
+                                 const GradPtrs& g, const LaunchCfg& L, cudaStream_t st);                         \
   cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI,           \
                           void* buf, const GradPtrs& g, const LaunchCfg& L, cudaStream_t st);                     \
   cudaError_t launch_collect(const DevScene& S, const KParams& kp, const float* dI, float tfloor, float* feats,   \
                              float* targets, int64_t cap, unsigned long long* count, const LaunchCfg& L,          \
                              cudaStream_t st);                                                                    \
+  /* sum of the copies of the albedo gradient, added to d_albedo (KParams::rep) */                                 \
+  cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,      \
+                             cudaStream_t st);                                                                     \
   cudaError_t launch_film_l2(const float* I, const float* T, int64_t n, float* dI, float* loss, int sms,          \
                              cudaStream_t st);                                                                    \
   cudaError_t launch_bidir(const DevScene& S, const KParams& kp, const BidirArgs& ba, bool backward, float* image, \
