@@ -45,15 +45,14 @@ struct BatchSpan {
 };
 
 // Kernel of a batched launch: the fused LRB-3 kernel, or its two-kernel form (pass 2,
-// with or without the primal's validity masks, then pass 3).
+// with or without the primal's validity masks; pass 3 runs over spans).
 enum BatchPass {
   BPASS_PRIMAL = 0,
   BPASS_PRIMAL_RES = 1,
   BPASS_LRB3 = 2,
   BPASS_RESLRB = 3,
   BPASS_LRB3_P2 = 4,
-  BPASS_LRB3_P2_MASK = 5,
-  BPASS_LRB3_P3 = 6
+  BPASS_LRB3_P2_MASK = 5
 };
 
 // `chains`: some attached item's scene has dielectrics (compiles the specular-chain variant).

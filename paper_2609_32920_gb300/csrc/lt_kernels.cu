@@ -831,34 +831,42 @@ __device__ __forceinline__ float3 tex_pos_adjoint(const float* albedo, int4 m, c
   return (cross(P.e2, mm) * gs + cross(mm, P.e1) * gt) * inv;
 }
 
-// Flush a vertex's completed adjoint: attached vertices map through their surface
-// coordinates, sliding ones run the chain's reverse sweep (their normal is explicit).
-template <bool CH, class H>
-__device__ __forceinline__ void pend_flush(const DevScene& S, const KParams& kp, uint64_t n, const PendAdj& p,
+// Flush a vertex's completed adjoint: attached vertices map through their surface coordinates,
+// sliding ones (their normal is explicit) need the chain's reverse sweep: true when the caller has
+// to run it (pend_sweep).  The sweep is large code; a kernel has it in one place, inlined into
+// each of three flushes it was over half of the specular-chain kernels' code, and ran on the few
+// lanes that complete a vertex at a step.  With the sweeps of a warp run together, the ResLRB
+// backward of the slab box went from 5.70 to 3.65 ms, the attached pass 3 of the caustic with
+// 65 537 paths from 311 to 280 us.
+template <bool CH>
+__device__ __forceinline__ bool pend_flush(const DevScene& S, const PendAdj& p, float* dh) {
+  if (!dh || p.prim < 0) return false;
+  const bool sl = CH && p.sliding;
+  scatter_heights(S, dh, p.prim, sl ? 0.0f : p.b1, sl ? 0.0f : p.b2, sl ? f3(0, 0, 0) : p.gx, p.gn);
+  return sl;
+}
+template <class H>
+__device__ __forceinline__ void pend_sweep(const DevScene& S, const KParams& kp, uint64_t n, const PendAdj& p,
                                            float* dh, const ChainCache* cc, const H& hits) {
-  if (!dh || p.prim < 0) return;
-  if (!CH || !p.sliding) {
-    scatter_heights(S, dh, p.prim, p.b1, p.b2, p.gx, p.gn);
-  } else {
-    scatter_heights(S, dh, p.prim, 0.0f, 0.0f, f3(0, 0, 0), p.gn);
-    propagate_sliding(S, kp, n, p.chain, p.k, p.gx, dh, cc, p.prim, hits);
-  }
+  propagate_sliding(S, kp, n, p.chain, p.k, p.gx, dh, cc, p.prim, hits);
 }
 
 // Attached bookkeeping on arrival at vertex k, before its own terms: the attached segment
 // weight with the anchor (weight lam_seg) completes the anchor's adjoint; an attached
 // specular vertex starts a chain (its Fresnel factors weigh lam_chain); a non-specular
-// vertex becomes the new pending anchor (sliding when it ends a chain).
+// vertex becomes the new pending anchor (sliding when it ends a chain).  True when the anchor's
+// adjoint needs its chain's sweep: the anchor is then in `pf` (and no longer in pv).
 // CH = false compiles the variant for scenes without dielectrics (no chains exist).
-template <bool CH, class H>
-__device__ __forceinline__ void att_enter(const DevScene& S, const KParams& kp, uint64_t n, int k, const Vtx& v,
-                                          float lam_seg, float lam_chain, PendAdj& pv, ChainInfo& chain,
-                                          float* dh, const ChainCache* cc, const H& hits) {
+template <bool CH>
+__device__ __forceinline__ bool att_enter(const DevScene& S, int k, const Vtx& v, float lam_seg, float lam_chain,
+                                          PendAdj& pv, ChainInfo& chain, float* dh, PendAdj& pf) {
+  bool sweep = false;
   if (!CH || v.attached) {
     PendAdj cur;
     pend_init(cur, v.prim, k, v.b1, v.b2, v.x, v.nraw);
     seg_adjoint(pv.x, pv.nr, v.x, v.nraw, lam_seg, pv.gx, pv.gn, cur.gx, cur.gn);
-    pend_flush<CH>(S, kp, n, pv, dh, cc, hits);
+    sweep = pend_flush<CH>(S, pv, dh);
+    if (CH && sweep) pf = pv;
     if (CH && !v.diffuse) {
       chain = chain_at(pv, k, v, lam_chain);
       scatter_heights(S, dh, v.prim, v.b1, v.b2, cur.gx, cur.gn);
@@ -871,6 +879,7 @@ __device__ __forceinline__ void att_enter(const DevScene& S, const KParams& kp, 
     pv.sliding = true;
     pv.chain = chain;
   }
+  return sweep;
 }
 
 // ======================================================================= learned target
@@ -1429,17 +1438,19 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
                       kp0.ticket + (MODE == 1 ? 0 : 1));
   else disp.init(kp0.n_paths);
   int jb = 0;
-  // FLUSH: the lane's path is done except the reverse sweep through the specular chain that
-  // ends at its pending vertex; with DEFER the sweep waits for other lanes of the warp
+  // FLUSH: the lane waits for the reverse sweep through the specular chain that ends at its
+  // completed vertex `pf`; the path goes on afterwards, or is done (flush_end), perhaps with
+  // another sweep from its last vertex (flush_pv)
   enum { IDLE = 0, PASS2 = 1, PASS3 = 2, FLUSH = 3 };
-  constexpr bool DEFER = CH && ATT && !BATCH && MODE != 1;
+  constexpr bool SWEEP = CH && ATT && MODE != 1;
+  bool flush_end = false, flush_pv = false;
   int phase = IDLE, k = 0, last = 0, nconn = 0;
   bool more = true;
   int64_t p = 0;
   Walk w;
   float3 dtot = f3(0, 0, 0), rem = f3(0, 0, 0);
   uint64_t valid = 0, known = 0;
-  PendAdj pv;
+  PendAdj pv, pf;
   ChainInfo chain;
   chain.ka = -1;
   pv.prim = -1;
@@ -1521,17 +1532,25 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     }
   };
   while (true) {
-    // A chain sweep at a path end is long and runs only on the lanes that end a path at that
-    // step.  With DEFER such a lane waits (FLUSH) until kFlushBatch lanes of its warp wait or
-    // the warp has nothing else to do, and the waiting lanes then sweep together.
-    if constexpr (DEFER) {
+    // A chain sweep is long and few lanes need one at a step: such a lane waits (FLUSH) until
+    // kFlushBatch lanes of its warp wait or the warp has nothing else to do, and the waiting
+    // lanes then sweep together.
+    if constexpr (SWEEP) {
       const unsigned fq = __ballot_sync(0xffffffffu, phase == FLUSH);
       if (fq) {
         const unsigned busy = __ballot_sync(0xffffffffu, phase == PASS2 || phase == PASS3 || (more && phase == IDLE));
         if (__popc(fq) >= kFlushBatch || busy == 0u) {
           if (phase == FLUSH) {
-            pend_flush<CH>(S0, kp0, (uint64_t)(kp0.path_offset + p), pv, gs.d_heights, &cc, log);
-            phase = IDLE;
+            const DevScene& S = BATCH ? ba.jobs[jb].S : S0;
+            const KParams& kp = BATCH ? ba.jobs[jb].kp : kp0;
+            float* dh = BATCH ? ba.jobs[jb].g.d_heights : gs.d_heights;
+            pend_sweep(S, kp, (uint64_t)(kp.path_offset + p), pf, dh, &cc, log);
+            if (flush_pv) {
+              pf = pv;
+              flush_pv = false;
+            } else {
+              phase = flush_end ? IDLE : PASS3;
+            }
           }
         }
       }
@@ -1667,7 +1686,12 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
         // attached segment weight and chain bookkeeping: every connection from here on
         // carries this vertex's factors, so they weigh the remaining adjoint before Eq. 16
-        if (att) att_enter<CH>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc, log);
+        bool sweep = false;
+        if (att) sweep = att_enter<CH>(S, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, pf);
+        if (SWEEP && sweep) {
+          phase = FLUSH;
+          flush_end = flush_pv = false;
+        }
         const bool rec_chain = CH && att && !v.diffuse;
         if (rec_chain) cc.record(chain, k, v, w.dir);
         float3 rho = f3(0, 0, 0);
@@ -1697,10 +1721,16 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         fin = k > last;
       }
       if (fin) {
-        if (DEFER && pv.prim >= 0 && pv.sliding && g.d_heights) {
+        const bool sweep = att && pend_flush<CH>(S, pv, g.d_heights);
+        if (SWEEP && phase == FLUSH) {  // the anchor's sweep is waiting already
+          flush_end = true;
+          flush_pv = sweep;
+        } else if (SWEEP && sweep) {
+          pf = pv;
           phase = FLUSH;
+          flush_end = true;
+          flush_pv = false;
         } else {
-          if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc, log);
           phase = IDLE;
         }
       }
@@ -1792,10 +1822,6 @@ template <bool MK>
 __global__ void __launch_bounds__(256) k_lrb3_p2_batch(BatchArgs ba) {
   lrb3_body<false, false, false, true, 1, MK>(ba.jobs[0].S, ba.jobs[0].kp, nullptr, ba.jobs[0].g, ba);
 }
-template <bool ATT, bool CH>
-__global__ void __launch_bounds__(256) k_lrb3_p3_batch(BatchArgs ba) {
-  lrb3_body<ATT, false, CH, true, 2>(ba.jobs[0].S, ba.jobs[0].kp, nullptr, ba.jobs[0].g, ba);
-}
 
 // Batched pass 3 by spans: a block takes the next span (one atomic by its first thread),
 // runs the single-scene pass-3 body over it with the item's shared-memory gradient sink,
@@ -1861,13 +1887,14 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
   if (BATCH) bdisp.init(); else disp.init(kp0.n_paths);
   int jb = 0;
   bool busy = false, more = true;
+  bool flush = false, flush_end = false, flush_pv = false;  // a chain sweep from pf waits (see lrb3_body)
   int64_t p = 0;
   int k = 0, R = 0;
   float3 P = f3(0, 0, 0);  // Lbar_R * S: the weight of every factor of L_R
   float lam = 0.0f;
   float2 q = make_float2(0.0f, 0.0f);
   Walk w;
-  PendAdj pv;
+  PendAdj pv, pf;
   ChainInfo chain;
   chain.ka = -1;
   pv.prim = -1;
@@ -1906,6 +1933,27 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     busy = true;
   };
   while (true) {
+    if constexpr (CH && ATT) {
+      const unsigned fq = __ballot_sync(0xffffffffu, flush);
+      if (fq) {
+        const unsigned rest = __ballot_sync(0xffffffffu, !flush && (busy || more));
+        if (__popc(fq) >= kFlushBatch || rest == 0u) {
+          if (flush) {
+            const DevScene& S = BATCH ? ba.jobs[jb].S : S0;
+            const KParams& kp = BATCH ? ba.jobs[jb].kp : kp0;
+            float* dh = BATCH ? ba.jobs[jb].g.d_heights : gs.d_heights;
+            pend_sweep(S, kp, (uint64_t)(kp.path_offset + p), pf, dh, &cc, log);
+            if (flush_pv) {
+              pf = pv;
+              flush_pv = false;
+            } else {
+              flush = false;
+              if (flush_end) busy = false;
+            }
+          }
+        }
+      }
+    }
     bool want = more && !busy;
     for (int draw = 0;; ++draw) {
       int jnew = jb;
@@ -1924,7 +1972,7 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     const KParams& kp = BATCH ? ba.jobs[jb].kp : kp0;
     const GradPtrs& g = BATCH ? ba.jobs[jb].g : gs;
     const bool att = ATT && (!BATCH || ba.jobs[jb].att);
-    const bool trav = busy && !w.dead;
+    const bool trav = busy && !flush && !w.dead;
     HitRec h;
     h.prim = -1;
     bool pending = false;
@@ -1938,7 +1986,7 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     }
     Vtx v;
     const bool alive = trav && !pending && walk_finish(S, w, h, v);
-    if (!busy || pending) continue;
+    if (!busy || flush || pending) continue;
     const uint64_t n = (uint64_t)(kp.path_offset + p);
     if (!alive) {  // the replay must reach the vertex the primal selected
       set_err(S, ERR_BOUNDS);
@@ -1947,7 +1995,10 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     }
     const float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
     if (CH) log.prim[k] = v.prim;
-    if (att) att_enter<CH>(S, kp, n, k, v, lam, lam, pv, chain, g.d_heights, &cc, log);
+    if (att && att_enter<CH>(S, k, v, lam, lam, pv, chain, g.d_heights, pf)) {
+      flush = true;
+      flush_end = flush_pv = false;
+    }
     const bool rec_chain = CH && att && !v.diffuse;
     if (rec_chain) cc.record(chain, k, v, w.dir);
     float3 ns = f3(0, 0, 0), rho = f3(0, 0, 0);
@@ -1965,8 +2016,17 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
     if (rec_chain) cc.record_branch(refl);
     walk_rr(kp, n, k, w);
     if (++k > R) {
-      if (att) pend_flush<CH>(S, kp, n, pv, g.d_heights, &cc, log);
-      busy = false;
+      const bool sweep = att && pend_flush<CH>(S, pv, g.d_heights);
+      if (flush) {  // the anchor's sweep is waiting already
+        flush_end = true;
+        flush_pv = sweep;
+      } else if (sweep) {
+        pf = pv;
+        flush = flush_end = true;
+        flush_pv = false;
+      } else {
+        busy = false;
+      }
     }
   }
   if (BATCH) {
@@ -1979,8 +2039,10 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
 
 // ResLRB backward (Sec. 4.2.1-4.2.2, Eq. 11-13): replay each path to its reservoir vertex R
 // and weight every factor of L_R with Lbar_R (.) S from the primal's record.
+// The specular-chain variant gains from resident warps like pass 3 does: learned target in the
+// slab box, 2 blocks of 128 threads per SM 3.65 ms, 4 3.79, 6 3.48, 8 4.07.
 template <bool ATT, bool CH>
-__global__ void __launch_bounds__(128) k_reslrb(DevScene S, KParams kp, const float* __restrict__ dI,
+__global__ void __launch_bounds__(128, CH ? 6 : 4) k_reslrb(DevScene S, KParams kp, const float* __restrict__ dI,
                                                 const float4* __restrict__ rec, GradPtrs g0) {
   reslrb_body<ATT, CH, false>(S, kp, dI, rec, g0, BatchArgs{});
 }
@@ -2744,7 +2806,7 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
     // ---- pass 3: the exact form's terms with each film position local, and the transport
     walk_start(S, kp.seed, n, Le, w, x0);
     float3 rem = dtot;
-    PendAdj pv;
+    PendAdj pv, pf;
     pend_init(pv, -1, -1, 0.0f, 0.0f, x0, S.ln);
     ChainInfo chain;
     chain.ka = -1;
@@ -2771,7 +2833,8 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
         }
       }
       const float4 r = rand4(kp.seed, n, (uint32_t)(k + 1));
-      att_enter<true>(S, kp, n, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, &cc, log);
+      if (att_enter<true>(S, k, v, hsum(rem), hsum(rem), pv, chain, g.d_heights, pf))
+        pend_sweep(S, kp, n, pf, g.d_heights, &cc, log);
       const bool rec_chain = !v.diffuse;
       if (rec_chain) cc.record(chain, k, v, w.dir);
       float3 ns = f3(0, 0, 0), rho = f3(0, 0, 0);
@@ -2810,7 +2873,7 @@ __global__ void __launch_bounds__(128) k_lrb3_literal(DevScene S, KParams kp, co
       pb = cur;
       pb.refl = refl;
     }
-    pend_flush<true>(S, kp, n, pv, g.d_heights, &cc, log);
+    if (pend_flush<true>(S, pv, g.d_heights)) pend_sweep(S, kp, n, pv, g.d_heights, &cc, log);
   }
   sink_end(kp, g0, sgrad);
   block_add3(g0.d_Le, gLe);
@@ -3002,11 +3065,6 @@ static int occupancy_of(K kern, int block) {
       break;                                                                     \
     case BPASS_LRB3_P2: CALL(k_lrb3_p2_batch<false>); break;                    \
     case BPASS_LRB3_P2_MASK: CALL(k_lrb3_p2_batch<true>); break;                \
-    case BPASS_LRB3_P3:                                                          \
-      if (att && chains) CALL((k_lrb3_p3_batch<true, true>));                    \
-      else if (att) CALL((k_lrb3_p3_batch<true, false>));                        \
-      else CALL((k_lrb3_p3_batch<false, false>));                                \
-      break;                                                                     \
     default:                                                                     \
       if (att && chains) CALL((k_reslrb_batch<true, true>));                     \
       else if (att) CALL((k_reslrb_batch<true, false>));                         \
