@@ -2094,8 +2094,10 @@ __global__ void __launch_bounds__(128) k_lrb2_reduce(DevScene S, KParams kp, con
 
 // ======================================================================= naive reverse
 // Reverse sweep over the per-vertex tape: suffix sums of Lbar_i L_i replace the replay.
+// Six blocks of 128 threads per SM: the sweep waits on its tape, caustic 2^20 paths 1.02 ms at the
+// compiler's own choice (3 blocks), 0.93 at 6, 0.95 at 8.
 template <bool ATT, bool CH>
-__global__ void __launch_bounds__(128) k_naive(DevScene S, KParams kp, const float* __restrict__ dI,
+__global__ void __launch_bounds__(128, 6) k_naive(DevScene S, KParams kp, const float* __restrict__ dI,
                                                const void* __restrict__ ws, GradPtrs g0) {
   extern __shared__ float sgrad[];
   const Sink sink = sink_begin(kp, g0, sgrad);
@@ -2212,8 +2214,12 @@ __device__ __forceinline__ float bidir_light_w(const DevScene& S, const BidirArg
 // Light side.  BWD = false: the primal (splat every weighted connection).  BWD = true: the
 // LRB-3 adjoint in one kernel per path (pass 2 accumulates delta_total, Eq. 14; pass 3
 // replays to the last valid connection, Eq. 15-17), detached.
+// Resident blocks: a path per thread leaves a warp waiting for its longest path, so more warps
+// help: box, 2^21 paths, adjoint 2.50 ms at the compiler's 4 blocks of 128, 2.33 at 6, 2.12 at 8;
+// primal 0.79, 0.76, 0.82.  The camera side likewise: adjoint 0.49, 0.48, 0.47, primal 0.19,
+// 0.18, 0.19.
 template <bool BWD>
-__global__ void __launch_bounds__(128) k_bidir_light(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
+__global__ void __launch_bounds__(128, BWD ? 8 : 6) k_bidir_light(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
                                                      const float* __restrict__ dI, GradPtrs g0) {
   extern __shared__ float sgrad[];
   GradPtrs g = g0;
@@ -2371,7 +2377,7 @@ __device__ __forceinline__ bool cam_vertex(const DevScene& S, const KParams& kp,
 // the sample's film position being fixed): a first walk sums the contributions, a replay
 // weights each vertex's albedo with the adjoint of the contributions from that vertex on.
 template <bool BWD>
-__global__ void __launch_bounds__(128) k_bidir_cam(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
+__global__ void __launch_bounds__(128, BWD ? 8 : 6) k_bidir_cam(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
                                                    const float* __restrict__ dI, GradPtrs g0) {
   extern __shared__ float sgrad[];
   GradPtrs g = g0;
