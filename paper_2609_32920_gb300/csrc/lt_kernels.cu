@@ -331,31 +331,32 @@ __device__ __forceinline__ void scatter_albedo(const DevScene& S, float* g, cons
 }
 
 // The same into copies of the albedo gradient (KParams::rep): every texture has 2^rep_bits
-// entries of 16 B, shared out equally over its texels (rounded up to a power of two), so that a
-// texture of one texel, which gets as many adds as one of 256, is spread as widely: the adds to an
-// address, and with them the rounding of its sum, stay few.  One 16-B reduction per texel.  A
+// entries of 16 B, shared out equally over its texels (rounded up to a power of two), at most
+// kRepCopies per texel, so that a texture of one texel, which gets as many adds as one of 256, has
+// about as many partial sums as there are resident blocks (each block's own sum in shared
+// memory is the other form, and the partial sums' rounding stays that one's: with 205 copies for
+// every texel, or thousands for a lone one, the box's gradient moved by 1e-5 to 2e-5).  One 16-B
+// reduction per texel.  A
 // shared-memory add of a float is a compare-and-swap loop that the warp waits for, twelve in a row
 // per vertex (335 us for 512 vertices per lane at 8 active lanes of 16 warps per SM); four
 // fire-and-forget vector reductions to copies in L2 take 233 us at the same rate and leave the
-// warp free.  Taps that fall on one texel (edges, one-texel textures) are added first.
+// warp free.
+constexpr int kRepCopies = 10;  // log2
 __device__ __forceinline__ int rep_copy_bits(int rep_bits, int texels) {  // log2 of a texel's copies
-  return rep_bits - (texels > 1 ? 32 - __clz(texels - 1) : 0);
+  return min(kRepCopies, rep_bits - (texels > 1 ? 32 - __clz(texels - 1) : 0));
 }
 __device__ __forceinline__ void scatter_albedo_rep(float4* rep, int rep_bits, int mat, int4 m, const TexFoot& f,
                                                    float3 wt, float3 rho) {
   float3 a = f3(wt.x / rho.x, wt.y / rho.y, wt.z / rho.z);
-  float w[4] = {f.w[0], f.w[1], f.w[2], f.w[3]};
-  if (f.idx[1] == f.idx[0]) { w[0] += w[1]; w[1] = 0.0f; w[2] += w[3]; w[3] = 0.0f; }
-  if (f.idx[2] == f.idx[0]) { w[0] += w[2]; w[2] = 0.0f; w[1] += w[3]; w[3] = 0.0f; }
   const int cb = rep_copy_bits(rep_bits, m.z * m.w);
   const unsigned lane = (blockIdx.x * blockDim.x + threadIdx.x) & ((1u << cb) - 1u);
   float4* base = rep + ((size_t)mat << rep_bits) + lane;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    if (w[k] == 0.0f) continue;
+    if (f.w[k] == 0.0f) continue;
     float4* p = base + ((size_t)((unsigned)(f.idx[k] - m.y) / 3u) << cb);
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(a.x * w[k]),
-                 "f"(a.y * w[k]), "f"(a.z * w[k]), "f"(0.0f)
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(a.x * f.w[k]),
+                 "f"(a.y * f.w[k]), "f"(a.z * f.w[k]), "f"(0.0f)
                  : "memory");
   }
 }
