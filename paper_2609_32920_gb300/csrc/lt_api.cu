@@ -367,6 +367,7 @@ KParams kparams(const lt_params* p, const lt_render_opts* o) {
   k.multi_n = nullptr;
   k.hits = HitBits{0, 0, 0, 0};
   k.order = nullptr;
+  k.order_n = nullptr;
   k.jac_noise = o->jac_noise;
   k.noise_seed = o->noise_seed;
   k.det_eps = o->det_eps > 0.0f ? o->det_eps : 1e-6f;
@@ -724,103 +725,6 @@ size_t lt_naive_workspace_bytes(const lt_render_opts* o) {
   return head + (size_t)o->n_paths * (size_t)o->max_depth * 32;
 }
 
-namespace {
-// Order of the plain primal's paths: a counting sort by the cell of the path's first direction
-// (64 x 64 cells of the two uniforms of the emitter's cosine sample, Eq. 2), so that the lanes
-// of a warp, and the warps running at the same time, trace first rays that leave in similar
-// directions, and so do their next few rays (measured on the caustic: cells of the emitter
-// point as well, 16 x 16 x 4 x 4 or 32 x 32 x 2 x 2, were slightly slower).  Every
-// path's result depends only on its index, so the order changes no result, only the
-// coherence of the traversals (and, through the path list, of LRB-3 passes 2 and 3).
-__device__ __forceinline__ int sort_key(uint64_t seed, uint64_t n) {
-  const float4 r = rand4(seed, n, 0);
-  const int a = min((int)(r.z * 64.0f), 63), b = min((int)(r.w * 64.0f), 63);
-  return a * 64 + b;
-}
-// Blocks of the sort: one per kSortPer paths up to kSortBlocks.  The counts are one row of
-// `blocks` entries per bin, so a small call clears, scans and reads back few entries.
-constexpr int64_t kSortPer = 4096;
-__host__ __device__ __forceinline__ int sort_blocks(int64_t n) {
-  const int64_t b = (n + kSortPer - 1) / kSortPer;
-  return (int)(b < 1 ? 1 : b < kSortBlocks ? b : kSortBlocks);
-}
-__device__ __forceinline__ int64_t sort_range(int64_t n, int blk) { return (n + gridDim.x - 1) / gridDim.x * blk; }
-// counts[bin][block] of the block's contiguous range of paths
-__global__ void __launch_bounds__(1024) k_sort_count(uint64_t seed, uint64_t off, int64_t n, unsigned* counts) {
-  __shared__ unsigned h[kSortBins];
-  for (int i = threadIdx.x; i < kSortBins; i += blockDim.x) h[i] = 0;
-  __syncthreads();
-  const int64_t lo = min(sort_range(n, blockIdx.x), n), hi = min(sort_range(n, blockIdx.x + 1), n);
-  for (int64_t p = lo + threadIdx.x; p < hi; p += blockDim.x) atomicAdd(&h[sort_key(seed, off + p)], 1u);
-  __syncthreads();
-  for (int i = threadIdx.x; i < kSortBins; i += blockDim.x) counts[(size_t)i * gridDim.x + blockIdx.x] = h[i];
-}
-// exclusive scan of counts in bin-major order: one warp per bin scans its row of `blocks`
-// entries, 32 at a time, then one block scans the bins' totals into the bin starts.  The rows
-// are read and written coalesced: 3 us for 256 blocks, where one thread per bin walking its
-// row took 80 us (a serial chain of 256 uncoalesced loads) whatever the number of paths.
-__global__ void __launch_bounds__(256) k_sort_rows(unsigned* counts, unsigned* totals, int blocks) {
-  const int bin = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (bin >= kSortBins) return;
-  unsigned* row = counts + (size_t)bin * blocks;
-  unsigned acc = 0;
-  for (int b0 = 0; b0 < blocks; b0 += 32) {
-    const int b = b0 + lane;
-    const unsigned v = b < blocks ? row[b] : 0u;
-    unsigned inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned u = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += u;
-    }
-    if (b < blocks) row[b] = acc + inc - v;
-    acc += __shfl_sync(0xffffffffu, inc, 31);
-  }
-  if (lane == 0) totals[bin] = acc;
-}
-__global__ void __launch_bounds__(1024) k_sort_bins(unsigned* totals) {
-  __shared__ unsigned wsum[32];
-  constexpr int per = kSortBins / 1024;
-  unsigned loc = 0;
-  for (int j = 0; j < per; ++j) loc += totals[threadIdx.x * per + j];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned inc = loc;
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += v;
-  }
-  if (lane == 31) wsum[wid] = inc;
-  __syncthreads();
-  if (wid == 0) {
-    const unsigned w = wsum[lane];
-    unsigned wi = w;
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += v;
-    }
-    wsum[lane] = wi - w;
-  }
-  __syncthreads();
-  unsigned run = wsum[wid] + inc - loc;
-  for (int j = 0; j < per; ++j) {
-    const unsigned c = totals[threadIdx.x * per + j];
-    totals[threadIdx.x * per + j] = run;
-    run += c;
-  }
-}
-// each block places its range's paths at bin start + its blocks-before offset + rank
-__global__ void __launch_bounds__(1024) k_sort_place(uint64_t seed, uint64_t off, int64_t n, const unsigned* counts,
-                                                     const unsigned* starts, uint32_t* order) {
-  __shared__ unsigned at[kSortBins];
-  for (int i = threadIdx.x; i < kSortBins; i += blockDim.x)
-    at[i] = starts[i] + counts[(size_t)i * gridDim.x + blockIdx.x];
-  __syncthreads();
-  const int64_t lo = min(sort_range(n, blockIdx.x), n), hi = min(sort_range(n, blockIdx.x + 1), n);
-  for (int64_t p = lo + threadIdx.x; p < hi; p += blockDim.x)
-    order[atomicAdd(&at[sort_key(seed, off + p)], 1u)] = (uint32_t)p;
-}
-}  // namespace
-
 lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, int est, float* image, void* aux,
                     size_t aux_bytes, void* stream) {
   lt_status v = check_opts(s, p, o);
@@ -848,19 +752,18 @@ lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, in
       kp.list = (uint32_t*)(base + lrb3_state_list(o->n_paths));
       kp.list_n = (unsigned long long*)(base + lrb3_state_count(o->n_paths));
       kp.ticket = kp.list_n + 1;  // the primal's chunk counter (the backward zeroes it again)
-      LT_CUDA(cudaMemsetAsync(kp.list_n, 0, 2 * sizeof(unsigned long long), st));
-      // the order of the paths (see sort_key)
-      uint32_t* order = (uint32_t*)(base + lrb3_state_order(o->n_paths));
-      unsigned* counts = (unsigned*)(base + lrb3_state_sort(o->n_paths));
-      unsigned* starts = counts + (size_t)kSortBins * kSortBlocks;
-      const uint64_t off = (uint64_t)o->path_offset;
-      const int nb = sort_blocks(o->n_paths);
-      k_sort_count<<<nb, 1024, 0, st>>>(o->seed, off, o->n_paths, counts);
-      k_sort_rows<<<kSortBins / 8, 256, 0, st>>>(counts, starts, nb);
-      k_sort_bins<<<1, 1024, 0, st>>>(starts);
-      k_sort_place<<<nb, 1024, 0, st>>>(o->seed, off, o->n_paths, counts, starts, order);
-      LT_CUDA(cudaGetLastError());
-      kp.order = order;
+      LT_CUDA(cudaMemsetAsync(kp.list_n, 0, 5 * sizeof(unsigned long long), st));
+      // the order of the paths, without those that end on their first ray; not when all paths
+      // start at once, one per resident lane or fewer (four blocks of 128 per SM), where its four
+      // launches cost more than it gives (2^14 paths of the small box 122 us a step with it, 99
+      // without; 2^16 of the caustic 528 and 506, of the box with heights 805 and 751; at 2^17 the
+      // caustic takes 549 and 566)
+      if (o->n_paths > (int64_t)s->sms * 4 * 128) {
+        kp.order = (uint32_t*)(base + lrb3_state_order(o->n_paths));
+        kp.order_n = kp.list_n + 4;
+        cudaError_t eo = launch_path_order(dev_for(s, o), kp, (unsigned*)(base + lrb3_state_sort(o->n_paths)), st);
+        if (eo) return fail(LT_ERR_CUDA, std::string("lt_primal: ") + cudaGetErrorString(eo));
+      }
     }
   }
   if (est == LT_EST_BUFFERED) kp.hits = hit_bits(s);

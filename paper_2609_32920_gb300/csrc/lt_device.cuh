@@ -113,6 +113,7 @@ __device__ __forceinline__ float3 cosine_dir(float3 n, float u0, float u1) {
   return t * (r * c) + b * (r * s) + n * sqrtf(fmaxf(0.0f, 1.0f - u0));
 }
 
+constexpr uint32_t kHashInit = 2166136261u;
 // FNV-1a over the four bytes of x.
 __device__ __forceinline__ void fnv(uint32_t& h, uint32_t x) {
 #pragma unroll
@@ -639,6 +640,25 @@ __device__ __forceinline__ bool occluded_w(const DevScene& S, float3 org, float3
 #ifndef LT_BVH_WIDTH
 #define LT_BVH_WIDTH 4
 #endif
+// Whether a ray meets the box of the whole BVH before tmax: false only when it enters no node.
+// The wide widths take the slab distances by the arithmetic of wide_boxes, which is monotone in
+// the planes, as is hit_box for the binary tree's own first test.
+__device__ __forceinline__ bool enters_bvh(const DevScene& S, float3 org, float3 dir, float tmax) {
+  if (S.n_nodes == 0) return false;
+  const float4 lo = __ldg(S.node), hi = __ldg(S.node + 1);
+  const float3 inv = safe_inv(dir);
+#if LT_BVH_WIDTH == 2
+  return hit_box(lo, hi, org, inv, tmax);
+#else
+  const float3 oi = f3(org.x * inv.x, org.y * inv.y, org.z * inv.z);
+  const bool nx = inv.x < 0.0f, ny = inv.y < 0.0f, nz = inv.z < 0.0f;
+  const float a = fmaxf(fmaxf(fmaf(nx ? hi.x : lo.x, inv.x, -oi.x), fmaf(ny ? hi.y : lo.y, inv.y, -oi.y)),
+                        fmaxf(fmaf(nz ? hi.z : lo.z, inv.z, -oi.z), 0.0f));
+  const float b = fminf(fminf(fmaf(nx ? lo.x : hi.x, inv.x, -oi.x), fmaf(ny ? lo.y : hi.y, inv.y, -oi.y)),
+                        fminf(fmaf(nz ? lo.z : hi.z, inv.z, -oi.z), tmax));
+  return a <= b;
+#endif
+}
 template <bool ST = false>
 __device__ __forceinline__ HitRec trace_closest(const DevScene& S, float3 org, float3 dir, int skip,
                                                 Census* cs = nullptr) {

@@ -17,6 +17,10 @@ cudaError_t launch_primal(const DevScene& S, const KParams& kp, int est, float* 
   return LT_BY_WIDTH(S.width, launch_primal(S, kp, est, image, aux, L, st));
 }
 
+cudaError_t launch_path_order(const DevScene& S, const KParams& kp, unsigned* area, cudaStream_t st) {
+  return LT_BY_WIDTH(S.width, launch_path_order(S, kp, area, st));
+}
+
 cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI,
                         const GradPtrs& g, void* state, bool mask_ready, const LaunchCfg& L, cudaStream_t st) {
   return LT_BY_WIDTH(S.width, launch_lrb3(S, kp, att, chains, dI, g, state, mask_ready, L, st));

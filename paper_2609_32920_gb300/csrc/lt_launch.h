@@ -32,7 +32,8 @@ struct KParams {
                                // (array lengths, or 0: that array goes to global memory directly)
   int priv_n;                  // n_alb + n_h: floats of dynamic shared memory per block
   const float* mlp;            // learned reservoir target parameters (DEVICE) or null (luminance)
-  const uint32_t* order;       // plain primal: the order in which it takes the paths (or null)
+  uint32_t* order;             // plain primal: the order in which it takes the paths (or null)
+  unsigned long long* order_n; // and how many are in it (the others ended on their first ray)
   void* vstate;                // plain primal: LRB-3 per-path state that receives each path's
                                // connection-validity mask (or null)
   int rr_depth;                // Russian roulette after vertices of depth >= rr_depth (0: off)
@@ -105,6 +106,8 @@ struct BidirArgs {
   cudaError_t launch_refit(const RefitArgs& a, cudaStream_t st);                                                  \
   cudaError_t launch_primal(const DevScene& S, const KParams& kp, int est, float* image, void* aux,               \
                             const LaunchCfg& L, cudaStream_t st);                                                 \
+  /* the plain primal's path order (KParams::order), `area`: the sort's work area of the state */                  \
+  cudaError_t launch_path_order(const DevScene& S, const KParams& kp, unsigned* area, cudaStream_t st);            \
   cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI,           \
                           const GradPtrs& g, void* state, bool mask_ready, const LaunchCfg& L, cudaStream_t st);  \
   cudaError_t launch_reslrb(const DevScene& S, const KParams& kp, bool att, bool chains, const float* dI,         \
@@ -146,7 +149,8 @@ LT_KERNEL_LAUNCHERS
 //  - the list of the paths that have a valid connection (uint32 indices relative to the call, at
 //    lrb3_state_list), written by the plain primal so that passes 2 and 3 visit only those, and
 //    256 B of counters at lrb3_state_count: its length, the passes' counters of entries taken
-//    (two), the number of listed paths with several connections (uint64 each);
+//    (two), the number of listed paths with several connections, the number of paths in the order
+//    (uint64 each); while the order is built, the list's place holds the paths' sort keys;
 //  - the order in which the plain primal takes the paths (uint32[n_paths] at lrb3_state_order;
 //    the backward reuses the array for the listed paths with several connections) and the
 //    counting sort's work area that builds it (kSortBins x kSortBlocks counts, then kSortBins
