@@ -651,9 +651,13 @@ lt_status lt_scene_create(const lt_scene_desc* d, void* stream, lt_scene** out) 
     collapse_wide(B, W, nd, flat_of, codes, wmap);
     const int nw = (int)codes.size() / W;
     s->n_wnodes[k] = nw;
-    std::vector<float> wn((size_t)nw * 8 * W, 0.0f);  // boxes are written by the refit
+    std::vector<float> wn((size_t)nw * 8 * W, 0.0f);  // the children's boxes are written by the refit
     for (int j = 0; j < nw; ++j)
-      for (int c = 0; c < W; ++c) std::memcpy(&wn[(size_t)j * 8 * W + 6 * W + c], &codes[j * W + c], 4);
+      for (int c = 0; c < W; ++c) {
+        float* slot = &wn[(size_t)j * 8 * W + c];
+        std::memcpy(slot + 6 * W, &codes[j * W + c], 4);
+        for (int q = 0; q < 6 && codes[j * W + c] == -1; ++q) slot[q * W] = q < 3 ? 3e38f : -3e38f;  // no ray enters
+      }
     if (nw > 0) {
       e = up((void**)&s->d_wnode[k], wn.data(), wn.size() * sizeof(float));
       if (!e) e = up((void**)&s->d_wmap[k], wmap.data(), wmap.size() * sizeof(int));
