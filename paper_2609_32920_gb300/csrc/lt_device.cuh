@@ -336,7 +336,7 @@ __device__ __forceinline__ bool occluded2(const DevScene& S, float3 org, float3 
 
 // ------------------------------------------------------------------ wide BVH traversal
 // A visit pushes at most W - 1 <= 7 entries.  The depth is checked once a visit and not at each
-// push (2^24 box paths: 8.56 -> 8.33 ms): with room for 8 more entries than may wait when a
+// push (2^22 box paths: 8.56 -> 8.33 ms): with room for 8 more entries than may wait when a
 // visit begins, its pushes stay inside the stack.
 constexpr int kWideStack = 64;
 constexpr int kWideStackRoom = kWideStack + 8;
@@ -385,7 +385,7 @@ __device__ __forceinline__ void wide_boxes(const DevScene& S, int j, float3 inv,
     const float a = fmaxf(fmaxf(txn, tyn), fmaxf(tzn, 0.0f));
     const float b = fminf(fminf(txf, tyf), fminf(tzf, tmax));
     // An empty slot (code -1) stores the inverted box (3e38, -3e38): a ray with a finite origin
-    // enters it beyond where it leaves it, so the slot needs no test of its own (2^24 box paths:
+    // enters it beyond where it leaves it, so the slot needs no test of its own (2^22 box paths:
     // 8.56 -> 8.37 ms).  A ray that is not finite may enter it, which only ends its search early
     // (-1 is kCodeDone), and such a ray meets no primitive.
     tn[c] = a <= b ? a : __int_as_float(0x7f800000);
@@ -417,7 +417,7 @@ __device__ __forceinline__ void sort_children(float k[W], int c[W]) {
 // with their entry distance, so the nearest is visited next and entries beyond the
 // current hit are dropped when popped.  Leaves are tested in a separate loop (while-while
 // form) so that a warp tests its lanes' pending leaves together.  The nearest child would be
-// popped at once, so it becomes the next entry without going over the stack (2^24 box paths:
+// popped at once, so it becomes the next entry without going over the stack (2^22 box paths:
 // 8.82 -> 8.56 ms; also a register for the entry on top of the stack: 8.77).  A stack overflow
 // (a tree deeper than the stack allows) drops entries and sets ERR_BOUNDS.
 //
@@ -682,8 +682,8 @@ __device__ __forceinline__ HitRec trace_closest(const DevScene& S, float3 org, f
 #endif
 }
 // Resumable closest hit (see TravState): the binary BVH finishes in the first call.
-// node and leaf visits per lane per step (caustic primal of 2^24 paths / box primal of 2^22: 5 4.82 /
-// 9.14 ms, 8 4.77 / 9.1, 10 4.54 / 9.04, 12 4.45 / 9.14, 16 4.44 / 9.47)
+// node and leaf visits per lane per step (caustic primal of 2^24 paths / box primal of 2^22: 8 3.88 /
+// 8.06 ms, 10 3.65 / 8.04, 14 3.56 / 8.25, 20 3.58 / 8.71)
 constexpr int kTraceBudget = 10;
 template <bool ST = false>
 __device__ __forceinline__ void trace_begin(const DevScene& S, float3 org, float3 dir, int skip, TravState& T,

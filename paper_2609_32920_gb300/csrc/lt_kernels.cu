@@ -553,12 +553,17 @@ __device__ __forceinline__ HitRec hit_known(const DevScene& S, float3 org, float
 // (a position adjoint continues into it when the current chain's anchor ends it), of at
 // most kChainCache vertices each; a longer or older chain is replayed as before.  The
 // states are the ones the replay would compute, from the same arithmetic.
-constexpr int kChainCache = 4;
+// A replay of c vertices intersects c(c+1)/2 primitives while the warp's other lanes wait, so
+// the cache holds the chains of a closed dielectric with many internal reflections too (learned
+// slab-box ResLRB adjoint at 4, 8, 12, 16, 24, 32 vertices: 3.37, 3.16, 3.03, 3.00, 2.89, 2.91 ms;
+// 65537 caustic paths of depth 13, whole step: 541, 546, 449, 449, 452 us at 4, 8, 12, 16, 24; 2^24
+// caustic paths, pass 3: 2.25, 2.18, 2.19, 2.20, 2.20 ms).  At most 32: `refl` has a bit each.
+constexpr int kChainCache = 24;
 constexpr int kDraws = 4;  // path draws per lane and step of the LRB-3 loop
-// lanes of a warp beyond their recorded hits that search together (box pass 3: 1 6.04 ms, 6 4.65,
-// 12 4.55, 20 5.16)
+// lanes of a warp beyond their recorded hits that search together (2^22 box paths, pass 3: 1 6.04 ms,
+// 6 4.65, 12 4.55, 20 5.16; with the shorter visits 8 3.00, 12 2.96, 16 3.11)
 constexpr int kSearchBatch = 12;
-constexpr int kFlushBatch = 16;  // waiting lanes of a warp that sweep their chains together (swept 8-24)
+constexpr int kFlushBatch = 16;  // waiting lanes of a warp that sweep their chains together (12 to 20: within 1 %)
 struct ChainRec {
   ChainInfo info;
   int len;  // recorded specular vertices info.ka .. info.ka+len-1; -1: not usable
