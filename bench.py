@@ -248,10 +248,11 @@ class Step:
     order of the paths (a counting sort, 4 kernels) and primal light tracing storing the
     paths' connection-validity masks and first connections (1 kernel), film L2 loss and image
     adjoint (1), LRB-3-pass backward in its three-pass form, attached (pass 2 of the
-    single-connection paths, pass 2 of the others, pass 3: 3 kernels).  Events around the
-    primal (with its sort) and the backward time them on the launching stream."""
+    single-connection paths, pass 2 of the others, pass 3 and the sum of its albedo copies: 4
+    kernels).  Events around the primal (with its sort) and the backward time them on the
+    launching stream."""
 
-    LAUNCHES = 14
+    LAUNCHES = 15
 
     def __init__(self, name, dev, path_offset=0, n_norm=0, n_paths=0, scatter=0):
         import torch
