@@ -263,8 +263,11 @@ __global__ void __launch_bounds__(1024) k_mlp_moments(const float* __restrict__ 
   __shared__ double sh[34];
   __shared__ double all[kMomBlocks][34];  // read in block 0
   if (threadIdx.x < 34) sh[threadIdx.x] = 0.0;
-  __syncthreads();
-  // thread = (row, quarter of its features): 16 B loads, and the targets with the first quarter
+  // a block may write to another one's shared memory only once that block is known to run: the
+  // barrier stands here, where the blocks are together anyway, and not before the write
+  cluster.sync();
+  // thread = (row, quarter of its features), four consecutive floats (the caller's arrays need no
+  // more than a float's alignment), and the targets with the first quarter
   const int q = threadIdx.x & 3;
   double a[5] = {}, b[5] = {};
   const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 4);
