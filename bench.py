@@ -440,7 +440,7 @@ def run_ours(args):
     peak_tflops = sms * 128 * 2 * sm_max * 1e6 / 1e12  # FP32 FMA lanes x 2 x max SM clock
     kernel_ms = {"primal": sum(primal_ms) / len(primal_ms), "lrb3_backward": sum(bwd_ms) / len(bwd_ms)}
     names = {"primal": "k_primal<PLAIN> (primal light tracing, sensor connections, splats, validity masks)",
-             "lrb3_backward": "k_lrb3_single + k_lrb3_p2 + k_lrb3_p3 (LRB-3 passes 2 and 3, attached)"}
+             "lrb3_backward": "k_lrb3_several + k_lrb3_p2 + k_lrb3_p3 (LRB-3 passes 2 and 3, attached)"}
     rooflines = {}
     for key in kernel_ms:
         ach = census[key]["flops"] / (kernel_ms[key] * 1e-3) / 1e12

@@ -138,7 +138,9 @@ typedef struct {
                            path_dbg rows are left as they are and not read), and
                            their replays intersect the recorded primitive at a
                            path's first vertices instead of searching the scene
-                           (the same hit bit for bit).                          */
+                           (the same hit bit for bit).  The backward leaves what the
+                           primal stored as it is: any number of calls may follow one
+                           primal, with other d_image, attached, scatter or path_dbg. */
   int rr_depth;         /* Russian roulette: after each vertex of depth >= rr_depth a
                            path continues with probability rr_prob (Philox stream 2
                            of that depth) and its throughput is divided by rr_prob;
@@ -473,7 +475,7 @@ lt_status lt_bidir_backward(lt_scene* scene, const lt_params* params, const lt_r
  * linear in max_depth) in `buffer`; this call computes delta_total = sum_i Lbar_i * L_i
  * from those records without tracing (Eq. 14) and then replays each path once to
  * backpropagate (Eq. 15-17), intersecting the primitives of its first vertices that the primal
- * kept (160 bits of a 40 B per-path record) and searching the scene beyond them.  Same
+ * kept (160 bits of a 40 B per-path record, 192 with max_depth <= 32) and searching the scene beyond them.  Same
  * result as lt_backward_lrb3.  buffer: DEVICE, lt_lrb2_buffer_bytes(opts) bytes, written
  * by lt_primal(LT_EST_BUFFERED) with the same opts (LT_ERR_OOM if smaller).  path_dbg
  * (optional) [n_paths][4] = (delta_total rgb, n valid connections). */
@@ -483,10 +485,11 @@ lt_status lt_backward_lrb2(lt_scene* scene, const lt_params* params, const lt_re
 size_t lt_lrb2_buffer_bytes(const lt_render_opts* opts);
 
 /* Bytes of the optional LRB-3 per-path state (opts->lrb3_state): a record of 32 B per path
- * (delta_total rgb; the primitives that the path's first vertices hit, as many as fit in 256
- * bits for pass 2 and in 160 for pass 3; for a path with exactly one valid connection its film
- * position and contribution, from which pass 2 takes delta_total instead of replaying the
- * path, and 96 bits of primitives), 8 B of validity bits and 4 B (the list of paths with a
+ * (for a path with several valid connections the primitives that its first vertices hit, as
+ * many as fit in 160 bits, and delta_total rgb once pass 2 has formed it; for a path with exactly
+ * one its film position and contribution, from which delta_total is taken instead of replaying
+ * the path, and 96 bits of primitives; with max_depth <= 32 half of the validity bits' place
+ * holds 32 more bits of primitives), 8 B of validity bits and 4 B (the list of paths with a
  * valid connection) per path, the list's length and the passes' counters (256 B), then 4 B
  * per path and a fixed 4.2 MB (the order in which the plain primal takes the paths, sorted by
  * the cell of each path's first direction, and the counting sort's work area; the order

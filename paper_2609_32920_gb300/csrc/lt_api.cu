@@ -375,10 +375,11 @@ KParams kparams(const lt_params* p, const lt_render_opts* o) {
 }
 
 // Primitives kept in the per-path records of a scene: as many bits as its largest index needs.
-HitBits hit_bits(const lt_scene* s) {
+HitBits hit_bits(const lt_scene* s, int max_depth) {
   int b = 1;
   while (b < 31 && (1ll << b) < s->n_prims) ++b;
-  return HitBits{b, std::min(256 / b, kMaxDepth), std::min(160 / b, kMaxDepth), std::min(96 / b, kMaxDepth)};
+  const int more = one_mask_word(max_depth) ? 32 : 0;
+  return HitBits{b, std::min((160 + more) / b, kMaxDepth), std::min((96 + more) / b, kMaxDepth), 1};
 }
 
 // Gradients accumulate per block in shared memory for each parameter array that fits in
@@ -749,7 +750,7 @@ lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, in
   KParams kp = kparams(p, o);
   if (est == LT_EST_PLAIN && o->lrb3_state) {
     kp.vstate = o->lrb3_state;
-    kp.hits = hit_bits(s);
+    kp.hits = hit_bits(s, o->max_depth);
     if (o->n_paths <= kListMaxPaths) {
       // the list of the paths with a valid connection, for LRB-3 passes 2 and 3
       char* base = (char*)o->lrb3_state;
@@ -770,7 +771,7 @@ lt_status lt_primal(lt_scene* s, const lt_params* p, const lt_render_opts* o, in
       }
     }
   }
-  if (est == LT_EST_BUFFERED) kp.hits = hit_bits(s);
+  if (est == LT_EST_BUFFERED) kp.hits = hit_bits(s, o->max_depth);
   cudaError_t e = launch_primal(dev_for(s, o), kp, est, image, aux, cfg_for(s, o), st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_primal: ") + cudaGetErrorString(e));
   return LT_OK;
@@ -798,7 +799,7 @@ lt_status lt_backward_lrb3(lt_scene* s, const lt_params* p, const lt_render_opts
   }
   // the primal recorded the primitives of each path's first vertices and, for a path with one
   // valid connection, that connection
-  if (o->lrb3_state && o->lrb3_mask_ready) kp.hits = hit_bits(s);
+  if (o->lrb3_state) kp.hits = o->lrb3_mask_ready ? hit_bits(s, o->max_depth) : HitBits{0, 0, 0, 1};
   if (o->lrb3_state && o->lrb3_mask_ready && o->n_paths <= kListMaxPaths) {
     // the primal listed the paths with a valid connection: passes 2 and 3 visit only those
     char* base = (char*)o->lrb3_state;
@@ -851,8 +852,9 @@ lt_status lt_backward_lrb2(lt_scene* s, const lt_params* p, const lt_render_opts
   if (o->n_paths == 0) return LT_OK;
   KParams kp = kparams(p, o);
   set_privatization(s, g, kp, o->scatter);
-  kp.hits = hit_bits(s);
-  kp.hits.cap1 = kp.hits.cap3;  // every record of the buffer has the wide form
+  kp.hits = hit_bits(s, o->max_depth);
+  kp.hits.cap1 = kp.hits.cap;  // every record of the buffer has the wide form, with delta_total
+  kp.hits.one = 0;
   const LaunchCfg L = cfg_for(s, o);
   cudaError_t e = launch_lrb2_reduce(dev_for(s, o), kp, dI, buf, gp, L, st);
   // the splat records are read: their place serves the copies of the albedo gradient
@@ -1143,7 +1145,7 @@ lt_status launch_group(lt_batch* b, int pass, const GroupLaunch& g, cudaStream_t
     // a resident grid, but no more blocks than spans
     const int64_t grid = std::min<int64_t>((int64_t)b->sms * g.per_sm, g.c1);
     cudaError_t e = launch_batch_spans(b->cfg.bvh_width, g.att, g.chains, b->d_jobs[table_of(b->cfg)],
-                                       b->d_spans[g.slot], (int)g.c1, ticket, block,
+                                       b->d_spans[g.slot], (int)g.c1, ticket, b->mask_ready, block,
                                        (int)std::max<int64_t>(grid, 1), b->span_smem, st);
     if (e) return fail(LT_ERR_CUDA, std::string("batched pass 3: ") + cudaGetErrorString(e));
     return LT_OK;
@@ -1295,7 +1297,7 @@ lt_status lt_batch_create(const lt_batch_item* items, int n, void* stream, lt_ba
     J.state = it.opts.lrb3_state;
     // the batched plain primal stores validity masks and hits there
     J.kp.vstate = it.opts.lrb3_state;
-    if (it.opts.lrb3_state && b->mask_ready) J.kp.hits = hit_bits(it.scene);
+    if (it.opts.lrb3_state) J.kp.hits = b->mask_ready ? hit_bits(it.scene, it.opts.max_depth) : HitBits{0, 0, 0, 1};
     set_privatization(it.scene, &it.grads, J.kp);  // used by pass 3 over spans only
     b->span_smem = std::max(b->span_smem, sizeof(float) * (size_t)J.kp.priv_n);
     J.att = it.opts.attached != 0;

@@ -64,8 +64,8 @@ enum BatchPass {
   int batch_occupancy(int pass, bool att, bool chains, int block);                                         \
   /* LRB-3 pass 3 over spans (see BatchSpan), `smem` bytes of gradient sink per block */                   \
   cudaError_t launch_batch_spans(bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans,      \
-                                 int n_spans, unsigned long long* ticket, int block, int grid, size_t smem, \
-                                 cudaStream_t st);                                                         \
+                                 int n_spans, unsigned long long* ticket, bool mask_ready, int block,       \
+                                 int grid, size_t smem, cudaStream_t st);                                  \
   int batch_spans_occupancy(bool att, bool chains, int block, size_t smem);
 namespace w2 { LT_BATCH_LAUNCHERS }
 namespace w4 { LT_BATCH_LAUNCHERS }
@@ -74,8 +74,8 @@ cudaError_t launch_batch(int width, int pass, bool att, bool chains, const Batch
                          cudaStream_t st);
 int batch_occupancy(int width, int pass, bool att, bool chains, int block);
 cudaError_t launch_batch_spans(int width, bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans,
-                               int n_spans, unsigned long long* ticket, int block, int grid, size_t smem,
-                               cudaStream_t st);
+                               int n_spans, unsigned long long* ticket, bool mask_ready, int block, int grid,
+                               size_t smem, cudaStream_t st);
 int batch_spans_occupancy(int width, bool att, bool chains, int block, size_t smem);
 
 }  // namespace lt

@@ -81,9 +81,10 @@ int batch_occupancy(int width, int pass, bool att, bool chains, int block) {
 }
 
 cudaError_t launch_batch_spans(int width, bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans,
-                               int n_spans, unsigned long long* ticket, int block, int grid, size_t smem,
-                               cudaStream_t st) {
-  return LT_BY_WIDTH(width, launch_batch_spans(att, chains, jobs, spans, n_spans, ticket, block, grid, smem, st));
+                               int n_spans, unsigned long long* ticket, bool mask_ready, int block, int grid,
+                               size_t smem, cudaStream_t st) {
+  return LT_BY_WIDTH(
+      width, launch_batch_spans(att, chains, jobs, spans, n_spans, ticket, mask_ready, block, grid, smem, st));
 }
 
 int batch_spans_occupancy(int width, bool att, bool chains, int block, size_t smem) {

@@ -510,7 +510,7 @@ struct TapeHits {
 // Primitives packed `bits` each into consecutive words (see HitBits), appended in vertex order:
 // the current word is in a register, full ones in the lane's local memory.
 struct HitPack {
-  uint32_t w[8];
+  uint32_t w[6];
   uint32_t acc;
   __device__ __forceinline__ void put(const HitBits& hb, int k, int prim) {
     if (k >= hb.cap) return;
@@ -1133,7 +1133,7 @@ __global__ void __launch_bounds__(1024) k_sort_count(DevScene S, KParams kp, uin
     if (!kp.census && first_ray_leaves(S, w.org, w.dir, w.skip)) {
       key = kSortEnded;
       ps.mlo[p] = 0u;
-      ps.mhi[p] = 0u;
+      if (!one_mask_word(kp.max_depth)) ps.mhi[p] = 0u;
       if (kp.hash) kp.hash[p] = kHashInit;
       if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     } else {
@@ -1391,15 +1391,15 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         const PathState ps = path_state(kp.vstate, kp.n_paths);
         const uint64_t vm = active ? vmask : 0ull;
         ps.mlo[p] = (uint32_t)vm;
-        ps.mhi[p] = (uint32_t)(vm >> 32);
+        if (!one_mask_word(kp.max_depth)) ps.mhi[p] = (uint32_t)(vm >> 32);
         if (vm) {
           hp.close(kp.hits, k);
           const bool one = (vm & (vm - 1)) == 0ull;
+          if (one_mask_word(kp.max_depth)) ps.mhi[p] = one ? hp.w[3] : hp.w[5];
           const float4 a = make_float4(__uint_as_float(hp.w[0]), __uint_as_float(hp.w[1]), __uint_as_float(hp.w[2]),
                                        one ? c1[0] : __uint_as_float(hp.w[3]));
           const float4 b = one ? make_float4(c1[1], c1[2], c1[3], c1[4])
-                               : make_float4(__uint_as_float(hp.w[4]), __uint_as_float(hp.w[5]),
-                                             __uint_as_float(hp.w[6]), __uint_as_float(hp.w[7]));
+                               : make_float4(__uint_as_float(hp.w[4]), 0.0f, 0.0f, 0.0f);
           ps.a[ps.step * p] = a;
           ps.b[ps.step * p] = b;
         }
@@ -1410,6 +1410,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         ps.a[ps.step * p] = make_float4(__uint_as_float(hp.w[0]), __uint_as_float(hp.w[1]),
                                         __uint_as_float(hp.w[2]), __uint_as_float(hp.w[3]));
         ps.b[ps.step * p].x = __uint_as_float(hp.w[4]);
+        if (one_mask_word(kp.max_depth)) ps.mhi[p] = hp.w[5];
       }
       if (EST == 2) ((int*)aux)[p] = active ? k : 0;
       if (EST == 3) ((int*)((char*)aux + lrb2_layout(kp.n_paths, kp.max_depth).counts))[p] = active ? k : 0;
@@ -1429,8 +1430,8 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
         ++nconn;
         L = mul(w.beta, rho) * (c.geo * kp.inv_n);
         if (REC && vmask == 0ull) {
-          // the path's first valid connection: LRB-3 pass 2 takes delta_total from its record
-          // when it stays the only one
+          // the path's first valid connection: the LRB-3 backward takes delta_total from its
+          // record when it stays the only one
           c1[0] = c.ux; c1[1] = c.uy; c1[2] = L.x; c1[3] = L.y; c1[4] = L.z;
         }
         vmask |= 1ull << k;
@@ -1519,11 +1520,21 @@ __global__ void __launch_bounds__(256) k_primal_batch(BatchArgs ba) {
   primal_body<EST, true>(ba.jobs[0].S, ba.jobs[0].kp, nullptr, nullptr, ba);
 }
 
+// Validity bits of a path.
+__device__ __forceinline__ uint64_t path_valid(const PathState& ps, int64_t p, int max_depth) {
+  return (uint64_t)ps.mlo[p] | (one_mask_word(max_depth) ? 0ull : (uint64_t)ps.mhi[p] << 32);
+}
 // delta_total of a path with one valid connection from its record (see lrb3_state_bytes).
 __device__ __forceinline__ float3 single_total(const DevScene& S, const KParams& kp, const float* dI, float4 a,
                                                float4 b) {
   const float3 L = f3(b.y, b.z, b.w);
   return mul(adjoint_read_f(dI, S.W, S.H, a.w, b.x, L, nullptr, kp.filter), L);
+}
+// delta_total into the record of a path with several: words 5-7 and nothing else of it.
+__device__ __forceinline__ void store_total(float4* b, float3 d) {
+  float* w = reinterpret_cast<float*>(b);
+  w[1] = d.x;
+  *reinterpret_cast<float2*>(w + 2) = make_float2(d.y, d.z);
 }
 
 // ======================================================================= LRB-3-pass
@@ -1541,16 +1552,20 @@ __device__ __forceinline__ float3 single_total(const DevScene& S, const KParams&
 // state (paths without a valid connection are skipped).
 // MK (MODE 1): the primal stored each path's validity mask, so pass 2 takes connection validity
 // from it, traces no visibility rays, stops after the last valid connection and skips paths
-// without one, and paths with one: k_lrb3_single forms their delta_total (a batch does it here).
+// without one, and paths with one: pass 3 forms delta_total = Lbar (.) L of those (Eq. 14) from the
+// recorded film position and contribution, the values a replay computes, and adds their
+// emitted-radiance gradient.
 // LOCAL: the calling block alone works on the path range (a span of a batch item).
 // With a path list (kp.list, masks known): MODE 1 (MK) visits only the listed paths with
 // several connections and MODE 2 the listed ones, so no lane draws a path it has nothing to do
 // for.
 // Known hits (kp.hits, from the primal's records): both passes intersect the recorded primitive
 // at a path's first vertices, which gives the search's hit bit for bit, and search the scene
-// only beyond them.  Box, 2^22 paths, depth 16 (11 bits a hit, 14 of
-// them in pass 3): pass 2 4.22 -> 1.24 ms, pass 3 7.62 -> 4.55 ms; caustic, 2^24 paths (16 bits):
-// pass 3 3.7 -> 2.65 ms, pass 2 0.27 -> 0.05 ms.
+// only beyond them.  Box, 2^22 paths, depth 16 (11 bits a hit): pass 2 4.22 ms searching, 1.23
+// with 17 recorded hits (192 bits); pass 3 2.94 ms with 14 (160 bits), 2.48 with 17.  Caustic, 2^24
+// paths (16 bits): pass 2 0.27 -> 0.05 ms, pass 3 3.7 -> 2.65 ms when the records came in.
+// Pass 3 takes delta_total of a path with one connection from its record instead of finding it
+// there: 2.20 -> 2.29 ms on the caustic (98 % of the listed paths), 0.14 -> 0.03 ms before it.
 template <bool ATT, bool ST, bool CH, bool BATCH, int MODE = 0, bool MK = false, bool LOCAL = false>
 __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0, const float* __restrict__ dI0,
                                           const GradPtrs& g0, const BatchArgs& ba, const PathState& st0 = {}) {
@@ -1600,8 +1615,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   constexpr bool LOG = CH || MODE == 0;
   HitLog log;
   constexpr bool HITS = MODE == 2 || (MODE == 1 && MK);
-  HitWords<MODE == 2 ? 5 : 8> hw;  // the path's recorded primitives, valid below vertex hcap
+  HitWords<6> hw;  // the path's recorded primitives, valid below vertex hcap
   int hcap = 0;
+  float c1[5];  // pass 2 without known masks: the first valid connection, for the record
   TravState ts;  // the lane's ray in flight (see TravState)
   LocalStack stk;
   bool inflight = false;
@@ -1614,19 +1630,26 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     if (got < 0) {
       more = false;
     } else if (MODE == 2) {
-      const uint64_t vm = (uint64_t)ps.mlo[got] | ((uint64_t)ps.mhi[got] << 32);
+      const uint64_t vm = path_valid(ps, got, kp.max_depth);
       if (vm && (!kp.mask || kp.mask[got])) {
         p = got;
         const float4 a = ps.a[ps.step * p], b = ps.b[ps.step * p];
-        if constexpr (MODE == 2) {
-          hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
-          hw.w[3] = __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x);
-          hcap = kp.hits.bits == 0 ? 0 : (vm & (vm - 1)) == 0ull ? kp.hits.cap1 : kp.hits.cap3;
-        }
+        const bool one = (vm & (vm - 1)) == 0ull;
+        hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
+        const uint32_t more = ps.mhi[p];
+        const bool narrow = one && kp.hits.one;  // words 3-7 are the connection
+        hw.w[3] = narrow ? more : __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = more;
+        hcap = narrow ? kp.hits.cap1 : kp.hits.cap;
         if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
         float3 x0;
         walk_start(S, kp.seed, (uint64_t)(kp.path_offset + p), Le, w, x0);
-        rem = f3(b.y, b.z, b.w);
+        if (narrow) {
+          rem = single_total(S, kp, dI0, a, b);
+          gLe = gLe + f3(rem.x / Le.x, rem.y / Le.y, rem.z / Le.z);  // emitted factor, weight delta_total
+          if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(rem.x, rem.y, rem.z, 1.0f);
+        } else {
+          rem = f3(b.y, b.z, b.w);
+        }
         valid = vm;
         pend_init(pv, -1, -1, 0.0f, 0.0f, x0, S.ln);
         chain.ka = -1;
@@ -1636,28 +1659,18 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         phase = PASS3;
       }
     } else if (!kp.mask || kp.mask[got]) {
-      if (MK) known = (uint64_t)ps.mlo[got] | ((uint64_t)ps.mhi[got] << 32);
+      if (MK) known = path_valid(ps, got, kp.max_depth);
       if (MK && !known) {  // no valid connection: delta_total = 0, the stored state stands
         if (kp.dbg) ((float4*)kp.dbg)[got] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         return;
       }
       if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
       if constexpr (MODE == 1 && MK) {
-        const bool one = (known & (known - 1)) == 0ull;
-        // one valid connection: k_lrb3_single has formed its delta_total without a replay
-        if (!BATCH && one) return;
+        if ((known & (known - 1)) == 0ull) return;  // one valid connection: pass 3 takes it from the record
         const float4 a = ps.a[ps.step * got], b = ps.b[ps.step * got];
-        if (one) {
-          const float3 d = single_total(S, kp, ba.jobs[jb].dI, a, b);
-          ps.b[ps.step * got] = make_float4(b.x, d.x, d.y, d.z);
-          gLe = gLe + f3(d.x / Le.x, d.y / Le.y, d.z / Le.z);
-          if (kp.dbg) ((float4*)kp.dbg)[got] = make_float4(d.x, d.y, d.z, 1.0f);
-          return;
-        }
         hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
-        hw.w[3] = __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = __float_as_uint(b.y);
-        hw.w[6] = __float_as_uint(b.z); hw.w[7] = __float_as_uint(b.w);
-        hcap = kp.hits.bits == 0 ? 0 : kp.hits.cap;
+        hw.w[3] = __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = ps.mhi[got];
+        hcap = kp.hits.cap;
       }
       p = got;
       float3 x0;
@@ -1780,9 +1793,12 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
           rho = tex_lookup(kp.albedo, v.m, v.b1, v.b2, nullptr);
           if (c.valid) {
             if (ST) ++nconns;
+            float3 L = mul(w.beta, rho) * (c.geo * kp.inv_n);
+            if (MODE == 1 && !MK && valid == 0ull) {
+              c1[0] = c.ux; c1[1] = c.uy; c1[2] = L.x; c1[3] = L.y; c1[4] = L.z;
+            }
             valid |= 1ull << k;
             ++nconn;
-            float3 L = mul(w.beta, rho) * (c.geo * kp.inv_n);
             float3 Lb = adjoint_read_f(dI, S.W, S.H, c.ux, c.uy, L, nullptr, kp.filter);
             dtot = dtot + mul(Lb, L);
           }
@@ -1796,12 +1812,17 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(dtot.x, dtot.y, dtot.z, (float)nconn);
         gLe = gLe + f3(dtot.x / Le.x, dtot.y / Le.y, dtot.z / Le.z);  // emitted factor, weight delta_total
         if (MODE == 1) {
-          if constexpr (MODE == 1) {
-            ps.b[ps.step * p] = make_float4(MK ? __uint_as_float(hw.w[4]) : 0.0f, dtot.x, dtot.y, dtot.z);
-            if (!MK) {
-              ps.mlo[p] = (uint32_t)valid;
-              ps.mhi[p] = (uint32_t)(valid >> 32);
+          if (!MK) {
+            ps.mlo[p] = (uint32_t)valid;
+            if (!one_mask_word(kp.max_depth)) ps.mhi[p] = (uint32_t)(valid >> 32);
+          }
+          if (!MK && (valid & (valid - 1)) == 0ull) {
+            if (valid) {  // the connection, as the primal records it
+              ps.a[ps.step * p].w = c1[0];
+              ps.b[ps.step * p] = make_float4(c1[1], c1[2], c1[3], c1[4]);
             }
+          } else {
+            store_total(ps.b + ps.step * p, dtot);
           }
           phase = IDLE;
         } else if (valid) {
@@ -1905,51 +1926,36 @@ __global__ void __launch_bounds__(128, 6) k_lrb3_p2(DevScene S, KParams kp, cons
                                                  PathState ps) {
   lrb3_body<false, ST, false, false, 1, MK>(S, kp, dI, g0, BatchArgs{}, ps);
 }
-// Pass 2 of the paths with exactly one valid connection (known masks, the primal's record of
-// the connection): delta_total = Lbar (.) L of that connection (Eq. 14) from its recorded film
-// position and contribution, the values a replay computes, one thread per listed path.  The
-// listed paths with several connections are collected for k_lrb3_p2.  On the caustic workload
-// 98 % of the paths with a connection have one.
-__global__ void __launch_bounds__(256) k_lrb3_single(DevScene S, KParams kp, const float* __restrict__ dI,
-                                                    GradPtrs g, PathState ps) {
+// The listed paths with several valid connections (known masks), for k_lrb3_p2; pass 3 needs no
+// pass 2 for the others.  On the caustic workload 98 % of the paths with a connection have one.
+__global__ void __launch_bounds__(256) k_lrb3_several(KParams kp, PathState ps) {
   const int64_t n = kp.list ? min((int64_t)*kp.list_n, kp.n_paths) : kp.n_paths;
-  const float3 Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
-  float3 gLe = f3(0, 0, 0);
   unsigned long long ones = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
     const int64_t i = base + threadIdx.x;
     const int64_t p = i < n ? (kp.list ? (int64_t)kp.list[i] : i) : -1;
     const bool in = p >= 0 && (!kp.mask || kp.mask[p]);
-    const uint64_t known = in ? (uint64_t)ps.mlo[p] | ((uint64_t)ps.mhi[p] << 32) : 0ull;
+    const uint64_t known = in ? path_valid(ps, p, kp.max_depth) : 0ull;
     const bool several = (known & (known - 1)) != 0ull;
-    if (kp.multi) {
-      const unsigned b = __ballot_sync(0xffffffffu, several);
-      if (b) {
-        const int lane = threadIdx.x & 31, leader = __ffs(b) - 1;
-        unsigned long long at = 0;
-        if (lane == leader) at = atomicAdd(kp.multi_n, (unsigned long long)__popc(b));
-        at = __shfl_sync(0xffffffffu, at, leader);
-        if (several) kp.multi[at + __popc(b & ((1u << lane) - 1u))] = (uint32_t)p;
-      }
+    const unsigned b = kp.multi ? __ballot_sync(0xffffffffu, several) : 0u;
+    if (b) {
+      const int lane = threadIdx.x & 31, leader = __ffs(b) - 1;
+      unsigned long long at = 0;
+      if (lane == leader) at = atomicAdd(kp.multi_n, (unsigned long long)__popc(b));
+      at = __shfl_sync(0xffffffffu, at, leader);
+      if (several) kp.multi[at + __popc(b & ((1u << lane) - 1u))] = (uint32_t)p;
     }
-    if (known == 0ull || several) continue;
-    const float4 a = ps.a[ps.step * p], r = ps.b[ps.step * p];
-    const float3 d = single_total(S, kp, dI, a, r);
-    ps.b[ps.step * p] = make_float4(r.x, d.x, d.y, d.z);
-    gLe = gLe + f3(d.x / Le.x, d.y / Le.y, d.z / Le.z);  // emitted factor, weight delta_total
-    ++ones;
-    if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(d.x, d.y, d.z, 1.0f);
+    if (known != 0ull && !several) ++ones;
   }
-  if (kp.census) {
+  if (kp.census) {  // connections that pass 2 does not visit
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ones += __shfl_xor_sync(0xffffffffu, ones, o);
     if ((threadIdx.x & 31) == 0 && ones) atomicAdd(kp.census + 4, ones);
   }
-  block_add3(g.d_Le, gLe);
 }
-
-// ... then pass 3 (albedo and height gradients) from that state.
+// ... then pass 3 from that state (albedo and height gradients; with known masks also the
+// emitted-radiance gradient of the paths with one connection).
 template <bool ATT, bool ST, bool CH>
 __global__ void __launch_bounds__(128, CH ? 8 : 4) k_lrb3_p3(DevScene S, KParams kp, const float* __restrict__ dI, GradPtrs g0,
                                                  PathState ps) {
@@ -1968,7 +1974,7 @@ __global__ void __launch_bounds__(256) k_lrb3_p2_batch(BatchArgs ba) {
 template <bool ATT, bool CH>
 __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restrict__ jobs,
                                                        const BatchSpan* __restrict__ spans, int n_spans,
-                                                       unsigned long long* ticket) {
+                                                       unsigned long long* ticket, bool mask_ready) {
   __shared__ int s_span;
   while (true) {
     if (threadIdx.x == 0) s_span = (int)atomicAdd(ticket, 1ull);
@@ -1989,7 +1995,7 @@ __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restric
     ps.mlo += span.start;
     ps.mhi += span.start;
     GradPtrs g = J.g;
-    g.d_Le = nullptr;  // pass 2 added the emitted-radiance gradient
+    if (!mask_ready) g.d_Le = nullptr;  // pass 2 added the whole emitted-radiance gradient
     const bool att = ATT && J.att;
     if (att) lrb3_body<ATT, false, CH, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
     else lrb3_body<false, false, false, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
@@ -2224,7 +2230,7 @@ __global__ void __launch_bounds__(128) k_lrb2_reduce(DevScene S, KParams kp, con
     float4* rec = ps.b + ps.step * p;
     rec->y = dtot.x; rec->z = dtot.y; rec->w = dtot.z;
     ps.mlo[p] = (uint32_t)valid;
-    ps.mhi[p] = (uint32_t)(valid >> 32);
+    if (!one_mask_word(kp.max_depth)) ps.mhi[p] = (uint32_t)(valid >> 32);
     gLe = gLe + f3(dtot.x / Le.x, dtot.y / Le.y, dtot.z / Le.z);  // emitted factor, weight delta_total
     if (kp.dbg) ((float4*)kp.dbg)[p] = make_float4(dtot.x, dtot.y, dtot.z, (float)nconn);
   }
@@ -3127,8 +3133,8 @@ cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool cha
     KParams k2 = kp;
     k2.priv_n = 0;  // pass 2 writes no albedo or height gradients
     GradPtrs g3 = g;
-    g3.d_Le = nullptr;  // pass 3 writes no emitted-radiance gradient
-    if (mask_ready) k_lrb3_single<<<L.sms * 4, 256, 0, st>>>(S, k2, dI, g, ps);
+    if (!mask_ready) g3.d_Le = nullptr;  // pass 2 adds the whole emitted-radiance gradient
+    if (mask_ready) k_lrb3_several<<<L.sms * 4, 256, 0, st>>>(k2, ps);
     if (kp.census) {
       if (mask_ready) launch_paths(k_lrb3_p2<true, true>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
       else launch_paths(k_lrb3_p2<true, false>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
@@ -3235,10 +3241,11 @@ cudaError_t launch_batch(int pass, bool att, bool chains, const BatchArgs& a, in
 }
 
 cudaError_t launch_batch_spans(bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans, int n_spans,
-                               unsigned long long* ticket, int block, int grid, size_t smem, cudaStream_t st) {
-  if (att && chains) k_lrb3_p3_spans<true, true><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket);
-  else if (att) k_lrb3_p3_spans<true, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket);
-  else k_lrb3_p3_spans<false, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket);
+                               unsigned long long* ticket, bool mask_ready, int block, int grid, size_t smem,
+                               cudaStream_t st) {
+  if (att && chains) k_lrb3_p3_spans<true, true><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
+  else if (att) k_lrb3_p3_spans<true, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
+  else k_lrb3_p3_spans<false, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
   return cudaGetLastError();
 }
 

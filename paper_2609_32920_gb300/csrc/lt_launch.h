@@ -8,11 +8,15 @@ namespace lt {
 struct DevScene;
 
 // Primitives of a path's first vertices as kept in its per-path record: `bits` each (enough for
-// the scene's primitives), at most `cap` of them for pass 2 (256 bits) and `cap3` for pass 3
-// (160 bits, or `cap1` in 96 bits for a path with one valid connection); see lrb3_state_bytes.
+// the scene's primitives), at most `cap` of them for a path with several valid connections and
+// `cap1` for one with one (160 and 96 bits, and 32 more where the validity bits need one word).
+// `one`: a path with one valid connection has that connection in its record (and not
+// delta_total); see lrb3_state_bytes.
 struct HitBits {
-  int bits, cap, cap3, cap1;
+  int bits, cap, cap1, one;
 };
+// Paths of at most 32 vertices need one word of validity bits; their second one holds hits.
+__host__ __device__ inline bool one_mask_word(int max_depth) { return max_depth <= 32; }
 
 // Per-call kernel parameters (by value).
 struct KParams {
@@ -45,7 +49,7 @@ struct KParams {
   unsigned long long* ticket;  // zeroed counters of entries taken: [0] pass 2, [1] pass 3 (plain
                                // primal with the LRB-3 state: [0] its 32-path chunks)
   uint32_t* multi;             // LRB-3 backward with a list: its paths with several connections
-  unsigned long long* multi_n; // (k_lrb3_single appends, pass 2 visits), and their number
+  unsigned long long* multi_n; // (k_lrb3_several appends, pass 2 visits), and their number
   HitBits hits;                // primitives kept in the per-path records (bits 0: none)
   float4* rep;                 // LRB-3 pass 3: copies of the albedo gradient, [material][2^rep_bits]
   int rep_bits;                // (see scatter_albedo_rep), or null
@@ -137,15 +141,19 @@ namespace w8 { LT_KERNEL_LAUNCHERS }
 LT_KERNEL_LAUNCHERS
 
 // `state` of launch_lrb3 (or null: fused kernel): per-path state of the two-kernel form.
-//  - a record of 32 B per path (at 0), eight words: words 5-7 are delta_total once pass 2 has
-//    formed it.  The plain primal keeps there, for a path with a valid connection, the
-//    primitives of its first vertices (HitBits, packed from bit 0 upwards), so that the passes
-//    intersect the known primitive instead of searching the scene: a path with several valid
-//    connections has words 0-7 for them until pass 2 writes delta_total and words 0-4 then; a
-//    path with one valid connection has words 0-2, and words 3-7 hold the film position and the
-//    contribution (u_x, u_y, L.rgb) of that connection.  One aligned sector per path, because
-//    the passes visit the paths in the order of the list and gather it.
-//  - validity bits 0-31 (at lrb3_state_mlo) and 32-63 (at lrb3_state_mhi), uint32 each;
+//  - a record of 32 B per path (at 0), eight words.  The plain primal keeps there, for a path
+//    with a valid connection, the primitives of its first vertices (HitBits, packed from bit 0
+//    upwards), so that the passes intersect the known primitive instead of searching the scene.
+//    A path with several valid connections has words 0-4 for them, and words 5-7 are pass 2's,
+//    for delta_total; a path with one has words 0-2, and words 3-7 hold the film position and the
+//    contribution (u_x, u_y, L.rgb) of that connection, from which pass 3 forms delta_total
+//    itself.  Pass 2 overwrites nothing that the primal recorded (where it traces the
+//    connections itself it writes the same one), so any number of backward calls, with other
+//    image adjoints, may follow one primal.  One aligned sector per path, because the passes
+//    visit the paths in the order of the list and gather it.
+//  - validity bits 0-31 (at lrb3_state_mlo) and 32-63 (at lrb3_state_mhi), uint32 each; with a
+//    depth of at most 32 the second word continues the recorded primitives instead (after word 2
+//    or word 4 of the record);
 //  - the list of the paths that have a valid connection (uint32 indices relative to the call, at
 //    lrb3_state_list), written by the plain primal so that passes 2 and 3 visit only those, and
 //    256 B of counters at lrb3_state_count: its length, the passes' counters of entries taken
