@@ -162,8 +162,8 @@ typedef struct {
                              not fit is added with plain global atomics, and so are the
                              splats; pass 3 of lt_backward_lrb3 with lrb3_mask_ready and
                              of lt_backward_lrb2 instead spreads the albedo gradient over
-                             copies in the state's (buffer's) then unused part and adds
-                             them up, where eight copies or more fit;
+                             copies in a work area of the state (buffer) and adds them
+                             up, where eight copies or more fit;
                            1 as 0, the per-block arrays up to the device's opt-in shared
                              memory per block (227 KB on GB300; fewer blocks may then be
                              resident per SM);
@@ -475,9 +475,11 @@ lt_status lt_bidir_backward(lt_scene* scene, const lt_params* params, const lt_r
  * linear in max_depth) in `buffer`; this call computes delta_total = sum_i Lbar_i * L_i
  * from those records without tracing (Eq. 14) and then replays each path once to
  * backpropagate (Eq. 15-17), intersecting the primitives of its first vertices that the primal
- * kept (160 bits of a 40 B per-path record, 192 with max_depth <= 32) and searching the scene beyond them.  Same
- * result as lt_backward_lrb3.  buffer: DEVICE, lt_lrb2_buffer_bytes(opts) bytes, written
- * by lt_primal(LT_EST_BUFFERED) with the same opts (LT_ERR_OOM if smaller).  path_dbg
+ * kept (160 bits of a 40 B per-path record, 192 with max_depth <= 32) and searching the scene
+ * beyond them.  Same result as lt_backward_lrb3.  buffer: DEVICE, lt_lrb2_buffer_bytes(opts)
+ * bytes (linear in max_depth, plus at most 4 MB for copies of the albedo gradient), written
+ * by lt_primal(LT_EST_BUFFERED) with the same opts (LT_ERR_OOM if smaller); any number of
+ * calls may follow one primal.  path_dbg
  * (optional) [n_paths][4] = (delta_total rgb, n valid connections). */
 lt_status lt_backward_lrb2(lt_scene* scene, const lt_params* params, const lt_render_opts* opts,
                            const float* d_image, void* buffer, size_t buffer_bytes, const lt_grads* grads,

@@ -857,9 +857,8 @@ lt_status lt_backward_lrb2(lt_scene* s, const lt_params* p, const lt_render_opts
   kp.hits.one = 0;
   const LaunchCfg L = cfg_for(s, o);
   cudaError_t e = launch_lrb2_reduce(dev_for(s, o), kp, dI, buf, gp, L, st);
-  // the splat records are read: their place serves the copies of the albedo gradient
   const Lrb2Layout lay = lrb2_layout(o->n_paths, o->max_depth);
-  v = e ? LT_OK : use_copies(s, g, o, (char*)buf + lay.rec4, std::min<size_t>(lay.recz - lay.rec4, 4u << 20), kp, st);
+  v = e ? LT_OK : use_copies(s, g, o, (char*)buf + lay.rep, lay.total - lay.rep, kp, st);
   if (v != LT_OK) return v;
   if (!e) e = launch_lrb2(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, buf, gp, L, st);
   if (!e && kp.rep) e = launch_rep_sum(s->dev, kp.rep, kp.rep_bits, s->n_mats, gp.d_albedo, st);

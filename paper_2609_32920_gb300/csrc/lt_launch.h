@@ -194,9 +194,11 @@ constexpr int64_t kListMaxPaths = 0xffffffffll;
 // Buffer of the buffered two-pass estimator (lrb_2pass): per path words 4-7 of an LRB-3 record
 // (16 B), validity bits 32-63 and its traced vertex count (int), then per vertex [depth][path]
 // the splat record (u_x, u_y, L.r, L.g) (float4; u_x < 0 = no valid connection) and L.b
-// (float), then per path words 0-3 of the record and validity bits 0-31.
+// (float), then per path words 0-3 of the record and validity bits 0-31, then the backward's
+// copies of the albedo gradient (at most 4 MB; the splat records stay as the primal wrote them, so
+// that any number of backward calls may follow it).
 struct Lrb2Layout {
-  size_t mhi, counts, rec4, recz, rec0, mlo, total;
+  size_t mhi, counts, rec4, recz, rec0, mlo, rep, total;
 };
 __host__ __device__ inline Lrb2Layout lrb2_layout(int64_t n, int d) {
   Lrb2Layout L;
@@ -206,7 +208,9 @@ __host__ __device__ inline Lrb2Layout lrb2_layout(int64_t n, int d) {
   L.recz = L.rec4 + align256((size_t)n * (size_t)d * 16);
   L.rec0 = L.recz + align256((size_t)n * (size_t)d * 4);
   L.mlo = L.rec0 + align256((size_t)n * 16);
-  L.total = L.mlo + align256((size_t)n * 4);
+  L.rep = L.mlo + align256((size_t)n * 4);
+  const size_t most = (size_t)4 << 20, rep = (size_t)n * (size_t)d * 16;
+  L.total = L.rep + align256(rep < most ? rep : most);
   return L;
 }
 __host__ __device__ inline PathState lrb2_path_state(void* buf, int64_t n, int d) {

@@ -58,6 +58,20 @@ def test_calls_after_one_primal(scene, depth, n, attached):
     assert (rows[0][:, 3] > 1).any() and (rows[0][:, 3] == 1).any()
 
 
+@pytest.mark.parametrize("scene,depth,n", [("box_3bit", 64, 4099), ("box_7bit", 12, 20011), ("slab_17bit", 12, 40001)])
+@pytest.mark.parametrize("attached", [0, 1])
+def test_buffered_calls_after_one_primal(scene, depth, n, attached):
+    S = lt.Scene(SCENES[scene]())
+    kw = dict(seed=9, n_paths=n, max_depth=depth, attached=attached)
+    o = S.opts(**kw)
+    buf = torch.empty(S.lrb2_buffer_bytes(o), dtype=torch.uint8, device="cuda")
+    S.primal(o, estimator=lt.EST_BUFFERED, aux=buf)
+    for k, scatter in [(1, 0), (2, 0), (3, 2), (1, 0)]:
+        dI = adjoint(S, k)
+        close(S.backward_lrb2(S.opts(scatter=scatter, **kw), dI, buf), S.backward_lrb3(o, dI))
+    S.sync_status()
+
+
 def batch_items(**kw):
     specs = [(I.box_scene(32), dict(n_paths=3000, max_depth=40, seed=1)),
              (I.box_scene(48, heightmap=8, hm_std=0.03), dict(n_paths=5001, max_depth=40, seed=2, attached=1)),
