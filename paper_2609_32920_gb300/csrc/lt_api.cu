@@ -1296,7 +1296,7 @@ lt_status lt_batch_create(const lt_batch_item* items, int n, void* stream, lt_ba
     J.state = it.opts.lrb3_state;
     // the batched plain primal stores validity masks and hits there
     J.kp.vstate = it.opts.lrb3_state;
-    if (it.opts.lrb3_state) J.kp.hits = b->mask_ready ? hit_bits(it.scene, it.opts.max_depth) : HitBits{0, 0, 0, 1};
+    if (it.opts.lrb3_state) J.kp.hits = hit_bits(it.scene, it.opts.max_depth);
     set_privatization(it.scene, &it.grads, J.kp);  // used by pass 3 over spans only
     b->span_smem = std::max(b->span_smem, sizeof(float) * (size_t)J.kp.priv_n);
     J.att = it.opts.attached != 0;

@@ -1995,7 +1995,10 @@ __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restric
     ps.mlo += span.start;
     ps.mhi += span.start;
     GradPtrs g = J.g;
-    if (!mask_ready) g.d_Le = nullptr;  // pass 2 added the whole emitted-radiance gradient
+    if (!mask_ready) {
+      g.d_Le = nullptr;               // pass 2 added the whole emitted-radiance gradient
+      kp.hits.cap = kp.hits.cap1 = 0;  // no primal need have recorded any
+    }
     const bool att = ATT && J.att;
     if (att) lrb3_body<ATT, false, CH, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
     else lrb3_body<false, false, false, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);

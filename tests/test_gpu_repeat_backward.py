@@ -102,6 +102,23 @@ def test_batched_pass_after_one_primal():
         check_batch(B.items)
 
 
+def test_batch_reads_a_state_of_a_batch_without_known_masks(monkeypatch):
+    """The primal pass records the same whatever the batch's own LRB-3 pass would use: here it is
+    run by a batch with an item that has no state, and read by one whose items all have."""
+    items = batch_items(lrb3_state=True)
+    B = lt.Batch(items + [dict(items[0], lrb3_state=False)])
+    B.run(lt.PASS_PRIMAL)
+    states = [it["_state"] for it in items]
+    second = batch_items(lrb3_state=True)
+    given = iter(states)
+    monkeypatch.setattr(lt.Scene, "new_lrb3_state", lambda self, n: next(given))
+    B2 = lt.Batch(second)
+    B2.run(lt.PASS_LRB3)
+    check_batch(second)
+    B.run(lt.PASS_LRB3)  # fused: some item has no state
+    check_batch(B.items)
+
+
 def test_tuned_pass_holds_one_complete_run():
     B = lt.Batch(batch_items(lrb3_state=True))
     B.run(lt.PASS_PRIMAL)
