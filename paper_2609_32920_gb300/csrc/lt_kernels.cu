@@ -1610,9 +1610,12 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   pv.prim = -1;
   ChainCache cc;
   cc.reset();
-  // primitives of the lane's path: pass 3 of the fused form replays along those of pass 2, and
-  // a chain's reverse sweep along those of the walk it ends
-  constexpr bool LOG = CH || MODE == 0;
+  // primitives of the lane's path, for a chain's reverse sweep; with chains, pass 3 of the fused form
+  // also replays along those of pass 2.  Without chains it searches again: lanes on their known
+  // hits would leave the warp's search to fewer lanes (fused, detached, known against searched: slab
+  // 2^22 paths 5.89 / 3.53 ms, box 2^20 paths 7.63 / 6.69, attached 9.72 / 8.63; with chains, slab in
+  // box 2^18 paths 7.30 / 7.58)
+  constexpr bool LOG = CH;
   HitLog log;
   constexpr bool HITS = MODE == 2 || (MODE == 1 && MK);
   HitWords<6> hw;  // the path's recorded primitives, valid below vertex hcap
@@ -1747,7 +1750,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         trav = false;
       }
     }
-    if (MODE == 0 && trav && phase == PASS3) {
+    if (MODE == 0 && CH && trav && phase == PASS3) {
       h = hit_known(S, w.org, w.dir, log(k));
     } else if (HITS && trav && k < hcap) {
       h = hit_known(S, w.org, w.dir, hw.get(kp.hits, k, S.n_prims));
