@@ -1129,7 +1129,8 @@ std::vector<GroupLaunch> plan_pass(const lt_batch* b, int pass) {
     if (g.c1 <= g.c0) continue;
     g.per_sm = b->cfg.blocks_per_sm > 0 ? b->cfg.blocks_per_sm
                : g.kpass == kSpanPass
-                   ? batch_spans_occupancy(b->cfg.bvh_width, g.att, g.chains, b->cfg.block_size, b->span_smem)
+                   ? batch_spans_occupancy(b->cfg.bvh_width, g.att, g.chains, b->mask_ready, b->cfg.block_size,
+                                           b->span_smem)
                    : batch_occupancy(b->cfg.bvh_width, g.kpass, g.att, g.chains, b->cfg.block_size);
     keep.push_back(g);
   }

@@ -66,7 +66,7 @@ enum BatchPass {
   cudaError_t launch_batch_spans(bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans,      \
                                  int n_spans, unsigned long long* ticket, bool mask_ready, int block,       \
                                  int grid, size_t smem, cudaStream_t st);                                  \
-  int batch_spans_occupancy(bool att, bool chains, int block, size_t smem);
+  int batch_spans_occupancy(bool att, bool chains, bool mask_ready, int block, size_t smem);
 namespace w2 { LT_BATCH_LAUNCHERS }
 namespace w4 { LT_BATCH_LAUNCHERS }
 namespace w8 { LT_BATCH_LAUNCHERS }
@@ -76,6 +76,6 @@ int batch_occupancy(int width, int pass, bool att, bool chains, int block);
 cudaError_t launch_batch_spans(int width, bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans,
                                int n_spans, unsigned long long* ticket, bool mask_ready, int block, int grid,
                                size_t smem, cudaStream_t st);
-int batch_spans_occupancy(int width, bool att, bool chains, int block, size_t smem);
+int batch_spans_occupancy(int width, bool att, bool chains, bool mask_ready, int block, size_t smem);
 
 }  // namespace lt

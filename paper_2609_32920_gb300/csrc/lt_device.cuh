@@ -697,11 +697,11 @@ __device__ __forceinline__ void trace_begin(const DevScene& S, float3 org, float
 }
 template <bool ST = false, class STK>
 __device__ __forceinline__ bool trace_resume(const DevScene& S, float3 org, float3 dir, int skip, TravState& T,
-                                             STK& stk, Census* cs = nullptr) {
+                                             STK& stk, int budget, Census* cs = nullptr) {
 #if LT_BVH_WIDTH == 2
   return true;
 #else
-  return trav_resume<LT_BVH_WIDTH, ST>(S, org, dir, skip, T, stk, kTraceBudget, cs);
+  return trav_resume<LT_BVH_WIDTH, ST>(S, org, dir, skip, T, stk, budget, cs);
 #endif
 }
 template <bool ST = false>

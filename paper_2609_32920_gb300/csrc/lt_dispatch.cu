@@ -87,8 +87,8 @@ cudaError_t launch_batch_spans(int width, bool att, bool chains, const BatchJob*
       width, launch_batch_spans(att, chains, jobs, spans, n_spans, ticket, mask_ready, block, grid, smem, st));
 }
 
-int batch_spans_occupancy(int width, bool att, bool chains, int block, size_t smem) {
-  return LT_BY_WIDTH(width, batch_spans_occupancy(att, chains, block, smem));
+int batch_spans_occupancy(int width, bool att, bool chains, bool mask_ready, int block, size_t smem) {
+  return LT_BY_WIDTH(width, batch_spans_occupancy(att, chains, mask_ready, block, smem));
 }
 
 }  // namespace lt

@@ -1304,7 +1304,7 @@ __device__ __forceinline__ void primal_body(const DevScene& S0, const KParams& k
     bool pending = false;  // the ray has visits left: the lane resumes it in the next step
     if (trav) {
       if (!inflight) trace_begin<ST>(S, w.org, w.dir, w.skip, ts, &cs);
-      inflight = !trace_resume<ST>(S, w.org, w.dir, w.skip, ts, stk, &cs);
+      inflight = !trace_resume<ST>(S, w.org, w.dir, w.skip, ts, stk, kTraceBudget, &cs);
       pending = inflight;
       h = ts.h;
     }
@@ -1555,6 +1555,9 @@ __device__ __forceinline__ void store_total(float4* b, float3 d) {
 // without one, and paths with one: pass 3 forms delta_total = Lbar (.) L of those (Eq. 14) from the
 // recorded film position and contribution, the values a replay computes, and adds their
 // emitted-radiance gradient.
+// MK (MODE 2): the plain or the buffered primal recorded hits.  Without (MK false) pass 3 has a
+// kernel of its own, which searches at every vertex: as a branch of the other the code for recorded
+// hits cost it a third (box 2^20 paths, attached 2.52 against 3.72 ms).
 // LOCAL: the calling block alone works on the path range (a span of a batch item).
 // With a path list (kp.list, masks known): MODE 1 (MK) visits only the listed paths with
 // several connections and MODE 2 the listed ones, so no lane draws a path it has nothing to do
@@ -1562,10 +1565,8 @@ __device__ __forceinline__ void store_total(float4* b, float3 d) {
 // Known hits (kp.hits, from the primal's records): both passes intersect the recorded primitive
 // at a path's first vertices, which gives the search's hit bit for bit, and search the scene
 // only beyond them.  Box, 2^22 paths, depth 16 (11 bits a hit): pass 2 4.22 ms searching, 1.23
-// with 17 recorded hits (192 bits); pass 3 2.94 ms with 14 (160 bits), 2.48 with 17.  Caustic, 2^24
-// paths (16 bits): pass 2 0.27 -> 0.05 ms, pass 3 3.7 -> 2.65 ms when the records came in.
-// Pass 3 takes delta_total of a path with one connection from its record instead of finding it
-// there: 2.20 -> 2.29 ms on the caustic (98 % of the listed paths), 0.14 -> 0.03 ms before it.
+// with 17 recorded hits (192 bits); pass 3 7.62 ms searching, 2.28 with 17.  Caustic, 2^24 paths
+// (16 bits): pass 2 0.27 -> 0.05 ms, pass 3 3.7 -> 2.21 ms.
 template <bool ATT, bool ST, bool CH, bool BATCH, int MODE = 0, bool MK = false, bool LOCAL = false>
 __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0, const float* __restrict__ dI0,
                                           const GradPtrs& g0, const BatchArgs& ba, const PathState& st0 = {}) {
@@ -1576,7 +1577,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     gs.d_albedo = sink.alb;
     gs.d_heights = sink.h;
   }
-  constexpr bool REP = MODE == 2 && !BATCH && !LOCAL;
+  constexpr bool REP = MODE == 2 && MK && !BATCH && !LOCAL;
   float3 Le = BATCH ? f3(0, 0, 0) : f3(kp0.Le[0], kp0.Le[1], kp0.Le[2]);
   float3 gLe = f3(0, 0, 0);
   Census cs = {0, 0, 0};
@@ -1617,7 +1618,11 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   // box 2^18 paths 7.30 / 7.58)
   constexpr bool LOG = CH;
   HitLog log;
-  constexpr bool HITS = MODE == 2 || (MODE == 1 && MK);
+  constexpr bool HITS = MODE != 0 && MK;
+  // a search of pass 3 without known hits goes on for 3 visits a step (box 2^20 paths, detached / slab
+  // 2^22 paths: 2 2.02 / 1.14 ms, 3 1.83 / 1.06, 4 1.81 / 1.22, 6 2.21 / 1.49, 10 2.64 / 1.57): its lanes
+  // stop at their path's last connection and take the next at different steps
+  constexpr int kBudget = MODE == 2 && !MK ? 3 : kTraceBudget;
   HitWords<6> hw;  // the path's recorded primitives, valid below vertex hcap
   int hcap = 0;
   float c1[5];  // pass 2 without known masks: the first valid connection, for the record
@@ -1638,11 +1643,13 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         p = got;
         const float4 a = ps.a[ps.step * p], b = ps.b[ps.step * p];
         const bool one = (vm & (vm - 1)) == 0ull;
-        hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
-        const uint32_t more = ps.mhi[p];
         const bool narrow = one && kp.hits.one;  // words 3-7 are the connection
-        hw.w[3] = narrow ? more : __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = more;
-        hcap = narrow ? kp.hits.cap1 : kp.hits.cap;
+        if constexpr (HITS) {
+          const uint32_t more = ps.mhi[p];
+          hw.w[0] = __float_as_uint(a.x); hw.w[1] = __float_as_uint(a.y); hw.w[2] = __float_as_uint(a.z);
+          hw.w[3] = narrow ? more : __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = more;
+          hcap = narrow ? kp.hits.cap1 : kp.hits.cap;
+        }
         if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
         float3 x0;
         walk_start(S, kp.seed, (uint64_t)(kp.path_offset + p), Le, w, x0);
@@ -1760,7 +1767,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
       if (trav) h = trace_closest<ST>(S, w.org, w.dir, w.skip, &cs);
     } else if (trav) {
       if (!inflight) trace_begin<ST>(S, w.org, w.dir, w.skip, ts, &cs);
-      inflight = !trace_resume<ST>(S, w.org, w.dir, w.skip, ts, stk, &cs);
+      inflight = !trace_resume<ST>(S, w.org, w.dir, w.skip, ts, stk, kBudget, &cs);
       pending = inflight;
       h = ts.h;
     }
@@ -1776,9 +1783,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     }
     // visibility only in pass 2; pass 3 reuses pass 2's validity bits (and with MK pass 2
     // reuses the primal's)
-    if (MK) {
+    if (MODE == 1 && MK) {
       if (phase == PASS2 && c.valid) c.valid = (known >> k) & 1ull;
-    } else {
+    } else if (MODE != 2) {
       const bool vis = phase == PASS2 && c.valid;
       if (vis && occluded<ST>(S, v.x, c.wc, c.dist, v.prim, &cs)) c.valid = false;
     }
@@ -1959,10 +1966,10 @@ __global__ void __launch_bounds__(256) k_lrb3_several(KParams kp, PathState ps) 
 }
 // ... then pass 3 from that state (albedo and height gradients; with known masks also the
 // emitted-radiance gradient of the paths with one connection).
-template <bool ATT, bool ST, bool CH>
+template <bool ATT, bool ST, bool CH, bool MK>
 __global__ void __launch_bounds__(128, CH ? 8 : 4) k_lrb3_p3(DevScene S, KParams kp, const float* __restrict__ dI, GradPtrs g0,
                                                  PathState ps) {
-  lrb3_body<ATT, ST, CH, false, 2>(S, kp, dI, g0, BatchArgs{}, ps);
+  lrb3_body<ATT, ST, CH, false, 2, MK>(S, kp, dI, g0, BatchArgs{}, ps);
 }
 
 // Batched two-kernel form: pass 2 over every item, then pass 3 per kernel group.
@@ -1974,10 +1981,10 @@ __global__ void __launch_bounds__(256) k_lrb3_p2_batch(BatchArgs ba) {
 // Batched pass 3 by spans: a block takes the next span (one atomic by its first thread),
 // runs the single-scene pass-3 body over it with the item's shared-memory gradient sink,
 // and flushes the sink into the item's arrays at the end of the span.
-template <bool ATT, bool CH>
+template <bool ATT, bool CH, bool MK>
 __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restrict__ jobs,
                                                        const BatchSpan* __restrict__ spans, int n_spans,
-                                                       unsigned long long* ticket, bool mask_ready) {
+                                                       unsigned long long* ticket) {
   __shared__ int s_span;
   while (true) {
     if (threadIdx.x == 0) s_span = (int)atomicAdd(ticket, 1ull);
@@ -1998,13 +2005,10 @@ __global__ void __launch_bounds__(256) k_lrb3_p3_spans(const BatchJob* __restric
     ps.mlo += span.start;
     ps.mhi += span.start;
     GradPtrs g = J.g;
-    if (!mask_ready) {
-      g.d_Le = nullptr;               // pass 2 added the whole emitted-radiance gradient
-      kp.hits.cap = kp.hits.cap1 = 0;  // no primal need have recorded any
-    }
+    if (!MK) g.d_Le = nullptr;  // pass 2 added the whole emitted-radiance gradient
     const bool att = ATT && J.att;
-    if (att) lrb3_body<ATT, false, CH, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
-    else lrb3_body<false, false, false, false, 2, false, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
+    if (att) lrb3_body<ATT, false, CH, false, 2, MK, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
+    else lrb3_body<false, false, false, false, 2, MK, true>(J.S, kp, J.dI, g, BatchArgs{}, ps);
   }
 }
 
@@ -2131,7 +2135,7 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
       if (trav) h = trace_closest(S, w.org, w.dir, w.skip);
     } else if (trav) {
       if (!inflight) trace_begin(S, w.org, w.dir, w.skip, ts);
-      inflight = !trace_resume(S, w.org, w.dir, w.skip, ts, stk);
+      inflight = !trace_resume(S, w.org, w.dir, w.skip, ts, stk, kTraceBudget);
       pending = inflight;
       h = ts.h;
     }
@@ -3149,13 +3153,17 @@ cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool cha
       else launch_paths(k_lrb3_p2<false, false>, L, kp.n_paths, 0, st, S, k2, dI, g, ps);
     }
     if (kp.census) {
-      if (att && chains) launch_paths(k_lrb3_p3<true, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-      else if (att) launch_paths(k_lrb3_p3<true, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-      else launch_paths(k_lrb3_p3<false, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      if (att && chains) launch_paths(k_lrb3_p3<true, true, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else if (att) launch_paths(k_lrb3_p3<true, true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else launch_paths(k_lrb3_p3<false, true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+    } else if (mask_ready) {
+      if (att && chains) launch_paths(k_lrb3_p3<true, false, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else if (att) launch_paths(k_lrb3_p3<true, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else launch_paths(k_lrb3_p3<false, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
     } else {
-      if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-      else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-      else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      if (att && chains) launch_paths(k_lrb3_p3<true, false, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else if (att) launch_paths(k_lrb3_p3<true, false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+      else launch_paths(k_lrb3_p3<false, false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
     }
     return cudaGetLastError();
   }
@@ -3201,9 +3209,9 @@ cudaError_t launch_lrb2(const DevScene& S, const KParams& kp, bool att, bool cha
   const size_t smem = kp.priv_n > 0 ? sizeof(float) * (size_t)kp.priv_n : 0;
   GradPtrs g3 = g;
   g3.d_Le = nullptr;  // added by the reduction
-  if (att && chains) launch_paths(k_lrb3_p3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-  else if (att) launch_paths(k_lrb3_p3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
-  else launch_paths(k_lrb3_p3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+  if (att && chains) launch_paths(k_lrb3_p3<true, false, true, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+  else if (att) launch_paths(k_lrb3_p3<true, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
+  else launch_paths(k_lrb3_p3<false, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g3, ps);
   return cudaGetLastError();
 }
 
@@ -3246,23 +3254,36 @@ cudaError_t launch_batch(int pass, bool att, bool chains, const BatchArgs& a, in
   return cudaGetLastError();
 }
 
+// Kernel of a batched pass 3 over spans.
+#define LT_SPANS_DISPATCH(CALL)                                \
+  if (mask_ready) {                                            \
+    if (att && chains) CALL((k_lrb3_p3_spans<true, true, true>));   \
+    else if (att) CALL((k_lrb3_p3_spans<true, false, true>));       \
+    else CALL((k_lrb3_p3_spans<false, false, true>));               \
+  } else {                                                     \
+    if (att && chains) CALL((k_lrb3_p3_spans<true, true, false>));  \
+    else if (att) CALL((k_lrb3_p3_spans<true, false, false>));      \
+    else CALL((k_lrb3_p3_spans<false, false, false>));              \
+  }
+
 cudaError_t launch_batch_spans(bool att, bool chains, const BatchJob* jobs, const BatchSpan* spans, int n_spans,
                                unsigned long long* ticket, bool mask_ready, int block, int grid, size_t smem,
                                cudaStream_t st) {
-  if (att && chains) k_lrb3_p3_spans<true, true><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
-  else if (att) k_lrb3_p3_spans<true, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
-  else k_lrb3_p3_spans<false, false><<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket, mask_ready);
+#define LT_LAUNCH_ONE(K) K<<<grid, block, smem, st>>>(jobs, spans, n_spans, ticket)
+  LT_SPANS_DISPATCH(LT_LAUNCH_ONE)
+#undef LT_LAUNCH_ONE
   return cudaGetLastError();
 }
 
-int batch_spans_occupancy(bool att, bool chains, int block, size_t smem) {
+int batch_spans_occupancy(bool att, bool chains, bool mask_ready, int block, size_t smem) {
   int n = 0;
-  cudaError_t e;
-  if (att && chains) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lrb3_p3_spans<true, true>, block, smem);
-  else if (att) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lrb3_p3_spans<true, false>, block, smem);
-  else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lrb3_p3_spans<false, false>, block, smem);
+  cudaError_t e = cudaSuccess;
+#define LT_OCC_ONE(K) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, block, smem)
+  LT_SPANS_DISPATCH(LT_OCC_ONE)
+#undef LT_OCC_ONE
   return e == cudaSuccess ? n : 0;
 }
+#undef LT_SPANS_DISPATCH
 
 int batch_occupancy(int pass, bool att, bool chains, int block) {
   int n = 0;
