@@ -2195,9 +2195,12 @@ __device__ __forceinline__ void reslrb_body(const DevScene& S0, const KParams& k
 // ResLRB backward (Sec. 4.2.1-4.2.2, Eq. 11-13): replay each path to its reservoir vertex R
 // and weight every factor of L_R with Lbar_R (.) S from the primal's record.
 // The specular-chain variant gains from resident warps like pass 3 does: learned target in the
-// slab box, 2 blocks of 128 threads per SM 3.65 ms, 4 3.79, 6 3.48, 8 4.07.
+// slab box, 2 blocks of 128 threads per SM 3.65 ms, 4 3.79, 6 3.48, 8 4.07.  The detached one too, a
+// little: box 2^20 / slab 2^22 / slab box 2^18 paths at 4, 5, 6, 8 blocks 0.617 / 0.694 / 0.330,
+// 0.583 / 0.617 / 0.339, 0.556 / 0.590 / 0.343, 0.539 / 0.545 / 0.395 ms; with the binary tree, slab 2^19
+// paths, 0.276, 0.242, 0.240, 0.257.
 template <bool ATT, bool CH>
-__global__ void __launch_bounds__(128, CH ? 6 : 4) k_reslrb(DevScene S, KParams kp, const float* __restrict__ dI,
+__global__ void __launch_bounds__(128, CH ? 6 : ATT ? 4 : 5) k_reslrb(DevScene S, KParams kp, const float* __restrict__ dI,
                                                 const float4* __restrict__ rec, GradPtrs g0) {
   reslrb_body<ATT, CH, false>(S, kp, dI, rec, g0, BatchArgs{});
 }
