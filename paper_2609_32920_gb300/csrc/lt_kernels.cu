@@ -2375,11 +2375,11 @@ __device__ __forceinline__ float bidir_light_w(const DevScene& S, const BidirArg
 // LRB-3 adjoint in one kernel per path (pass 2 accumulates delta_total, Eq. 14; pass 3
 // replays to the last valid connection, Eq. 15-17), detached.
 // Resident blocks: a path per thread leaves a warp waiting for its longest path, so more warps
-// help: box, 2^21 paths, adjoint 2.50 ms at the compiler's 4 blocks of 128, 2.33 at 6, 2.12 at 8;
-// primal 0.79, 0.76, 0.82.  The camera side likewise: adjoint 0.49, 0.48, 0.47, primal 0.19,
-// 0.18, 0.19.
+// help: box, 2^21 paths, adjoint 2.50 ms at the compiler's 4 blocks of 128, 2.33 at 6, 2.12 at 8; the
+// camera side likewise, 0.49, 0.48, 0.47.  The primals of both take 5 blocks, with which they spill
+// little: 2^18 paths and a third as many samples, together, 4 to 7 blocks 0.162, 0.146, 0.154, 0.157.
 template <bool BWD>
-__global__ void __launch_bounds__(128, BWD ? 8 : 6) k_bidir_light(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
+__global__ void __launch_bounds__(128, BWD ? 8 : 5) k_bidir_light(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
                                                      const float* __restrict__ dI, GradPtrs g0) {
   extern __shared__ float sgrad[];
   GradPtrs g = g0;
@@ -2537,7 +2537,7 @@ __device__ __forceinline__ bool cam_vertex(const DevScene& S, const KParams& kp,
 // the sample's film position being fixed): a first walk sums the contributions, a replay
 // weights each vertex's albedo with the adjoint of the contributions from that vertex on.
 template <bool BWD>
-__global__ void __launch_bounds__(128, BWD ? 8 : 6) k_bidir_cam(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
+__global__ void __launch_bounds__(128, BWD ? 8 : 5) k_bidir_cam(DevScene S, KParams kp, BidirArgs ba, float* __restrict__ image,
                                                    const float* __restrict__ dI, GradPtrs g0) {
   extern __shared__ float sgrad[];
   GradPtrs g = g0;
