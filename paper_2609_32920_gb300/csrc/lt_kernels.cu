@@ -1567,7 +1567,7 @@ __device__ __forceinline__ void store_total(float4* b, float3 d) {
 // only beyond them.  Box, 2^22 paths, depth 16 (11 bits a hit): pass 2 4.22 ms searching, 1.23
 // with 17 recorded hits (192 bits); pass 3 7.62 ms searching, 2.28 with 17.  Caustic, 2^24 paths
 // (16 bits): pass 2 0.27 -> 0.05 ms, pass 3 3.7 -> 2.21 ms.
-template <bool ATT, bool ST, bool CH, bool BATCH, int MODE = 0, bool MK = false, bool LOCAL = false>
+template <bool ATT, bool ST, bool CH, bool BATCH, int MODE = 0, bool MK = false, bool LOCAL = false, bool FEW = false>
 __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0, const float* __restrict__ dI0,
                                           const GradPtrs& g0, const BatchArgs& ba, const PathState& st0 = {}) {
   extern __shared__ float sgrad[];
@@ -1615,8 +1615,8 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   // also replays along those of pass 2.  Without chains it searches again: lanes on their known
   // hits would leave the warp's search to fewer lanes (fused, detached, known against searched: slab
   // 2^22 paths 5.89 / 3.53 ms, box 2^20 paths 7.63 / 6.69, attached 9.72 / 8.63; with chains, slab in
-  // box 2^18 paths 7.30 / 7.58)
-  constexpr bool LOG = CH;
+  // box 2^18 paths 7.30 / 7.58), except in small calls (FEW: see launch_lrb3)
+  constexpr bool LOG = CH || FEW;
   HitLog log;
   constexpr bool HITS = MODE != 0 && MK;
   // a search of pass 3 without known hits goes on for 3 visits a step (box 2^20 paths, detached / slab
@@ -1757,7 +1757,7 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
         trav = false;
       }
     }
-    if (MODE == 0 && CH && trav && phase == PASS3) {
+    if (MODE == 0 && LOG && trav && phase == PASS3) {
       h = hit_known(S, w.org, w.dir, log(k));
     } else if (HITS && trav && k < hcap) {
       h = hit_known(S, w.org, w.dir, hw.get(kp.hits, k, S.n_prims));
@@ -1921,9 +1921,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   block_add3(g0.d_Le, gLe);
 }
 
-template <bool ATT, bool ST, bool CH>
+template <bool ATT, bool ST, bool CH, bool FEW = false>
 __global__ void __launch_bounds__(128, 4) k_lrb3(DevScene S, KParams kp, const float* __restrict__ dI, GradPtrs g0) {
-  lrb3_body<ATT, ST, CH, false>(S, kp, dI, g0, BatchArgs{});
+  lrb3_body<ATT, ST, CH, false, 0, false, false, FEW>(S, kp, dI, g0, BatchArgs{});
 }
 
 // Two-kernel form: pass 2 (per-path state out, emitted-radiance gradient) ...
@@ -3177,7 +3177,14 @@ cudaError_t launch_lrb3(const DevScene& S, const KParams& kp, bool att, bool cha
     else if (att) launch_paths(k_lrb3<true, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g);
     else launch_paths(k_lrb3<false, true, false>, L, kp.n_paths, smem, st, S, kp, dI, g);
   } else {
+    // few: at most one warp per scheduler, whose longest path the call waits for; the second walk
+    // then goes along the known hits (known against searched: box of 4096 paths 0.306 / 0.336 ms, of
+    // 19456 0.333 / 0.364, of 30000 0.410 / 0.395, of 250000 1.44 / 1.37; slab, 19456 0.111 / 0.129, 60000
+    // 0.158 / 0.157)
+    const bool few = kp.n_paths <= (int64_t)L.sms * 128;
     if (att && chains) launch_paths(k_lrb3<true, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g);
+    else if (att && few) launch_paths(k_lrb3<true, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g);
+    else if (few) launch_paths(k_lrb3<false, false, false, true>, L, kp.n_paths, smem, st, S, kp, dI, g);
     else if (att) launch_paths(k_lrb3<true, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g);
     else launch_paths(k_lrb3<false, false, false>, L, kp.n_paths, smem, st, S, kp, dI, g);
   }
