@@ -334,11 +334,12 @@ __device__ __forceinline__ void scatter_albedo(const DevScene& S, float* g, cons
 
 // The same into copies of the albedo gradient (KParams::rep): every texture has 2^rep_bits
 // entries of 16 B, shared out equally over its texels (rounded up to a power of two), at most
-// kRepCopies per texel, so that a texture of one texel, which gets as many adds as one of 256, has
-// about as many partial sums as there are resident blocks (each block's own sum in shared
-// memory is the other form, and the partial sums' rounding stays that one's: with 205 copies for
-// every texel, or thousands for a lone one, the box's gradient moved by 1e-5 to 2e-5).  One 16-B
-// reduction per texel.  A
+// 2^kRepCopies per texel.  More copies are more partial sums and so a smaller rounding error; the cap
+// is there because a one-texel gradient with thousands of them left the per-block sums in shared
+// memory, the other form, by more than 2e-5 (the box; 1e-5 at the cap).  Error against an FP64 sum over
+// parts of the paths, per-block sums / copies: box with 16 x 16 textures 2^17 paths 3.8e-7 / 2.2e-7,
+// 2^19 4.8e-7 / 3.5e-7, 2^22 4.1e-7 / 3.0e-7, with one-texel textures 2^20 5.0e-7 / 3.9e-7, caustic 2^22
+// 2.2e-7 / 1.6e-7.  One 16-B reduction per texel.  A
 // shared-memory add of a float is a compare-and-swap loop that the warp waits for, twelve in a row
 // per vertex (335 us for 512 vertices per lane at 8 active lanes of 16 warps per SM); four
 // fire-and-forget vector reductions to copies in L2 take 233 us at the same rate and leave the
@@ -560,7 +561,7 @@ __device__ __forceinline__ HitRec hit_known(const DevScene& S, float3 org, float
 // caustic paths, pass 3: 2.25, 2.18, 2.19, 2.20, 2.20 ms).  At most 32: `refl` has a bit each.
 constexpr int kChainCache = 24;
 constexpr int kDraws = 4;  // path draws per lane and step of the LRB-3 loop
-// lanes of a warp beyond their recorded hits that search together (2^22 box paths, pass 3: 1 6.04 ms,
+// lanes of a warp beyond their recorded hits that search together (2^22 box paths, pass 3 with 14 hits: 1 6.04 ms,
 // 6 4.65, 12 4.55, 20 5.16; with the shorter visits 8 3.00, 12 2.96, 16 3.11)
 constexpr int kSearchBatch = 12;
 constexpr int kFlushBatch = 16;  // waiting lanes of a warp that sweep their chains together (12 to 20: within 1 %)
@@ -1545,8 +1546,8 @@ __device__ __forceinline__ void store_total(float4* b, float3 d) {
 // path takes the next one from its warp's range, in the same step as its last needed
 // vertex, drawing again over paths with nothing to trace.  The connection-validity bits
 // found in pass 2 are kept in a register mask so pass 3 traces no visibility rays.
-// BATCH: per-lane item (BatchDispenser), global gradient atomics, per-item attached flag;
-// S0, kp0, dI0 and g0 are not used.
+// BATCH (MODE 0 and 1): per-lane item (BatchDispenser), global gradient atomics, per-item attached
+// flag; S0, kp0, dI0 and g0 are not used.
 // MODE 0: passes 2 and 3 fused per lane.  MODE 1: pass 2 only, storing delta_total and the
 // validity mask of a path in its state (PathState).  MODE 2: pass 3 only, starting from that
 // state (paths without a valid connection are skipped).
@@ -1650,7 +1651,6 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
           hw.w[3] = narrow ? more : __float_as_uint(a.w); hw.w[4] = __float_as_uint(b.x); hw.w[5] = more;
           hcap = narrow ? kp.hits.cap1 : kp.hits.cap;
         }
-        if (BATCH) Le = f3(kp.Le[0], kp.Le[1], kp.Le[2]);
         float3 x0;
         walk_start(S, kp.seed, (uint64_t)(kp.path_offset + p), Le, w, x0);
         if (narrow) {
