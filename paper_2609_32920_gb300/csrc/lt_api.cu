@@ -365,6 +365,7 @@ KParams kparams(const lt_params* p, const lt_render_opts* o) {
   k.rep_bits = 0;
   k.multi = nullptr;
   k.multi_n = nullptr;
+  k.le_sum = nullptr;
   k.hits = HitBits{0, 0, 0, 0};
   k.order = nullptr;
   k.order_n = nullptr;
@@ -808,7 +809,9 @@ lt_status lt_backward_lrb3(lt_scene* s, const lt_params* p, const lt_render_opts
     kp.ticket = kp.list_n + 1;
     kp.multi_n = kp.list_n + 3;
     kp.multi = (uint32_t*)(base + lrb3_state_order(o->n_paths));
-    LT_CUDA(cudaMemsetAsync(kp.ticket, 0, 3 * sizeof(unsigned long long), st));
+    kp.le_sum = (double*)(kp.list_n + 5);
+    // the tickets, the number of paths with several connections, the primal's order length, le_sum
+    LT_CUDA(cudaMemsetAsync(kp.ticket, 0, 8 * sizeof(unsigned long long), st));
     // the sort's work area is free once the primal has run
     v = use_copies(s, g, o, base + lrb3_state_sort(o->n_paths),
                    lrb3_state_bytes(o->n_paths) - lrb3_state_sort(o->n_paths), kp, st);
@@ -816,7 +819,7 @@ lt_status lt_backward_lrb3(lt_scene* s, const lt_params* p, const lt_render_opts
   }
   cudaError_t e = launch_lrb3(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, gp,
                               o->lrb3_state, o->lrb3_state && o->lrb3_mask_ready, cfg_for(s, o), st);
-  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp.rep, kp.rep_bits, s->n_mats, gp.d_albedo, st);
+  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp, s->n_mats, gp, st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb3: ") + cudaGetErrorString(e));
   return LT_OK;
 }
@@ -861,7 +864,7 @@ lt_status lt_backward_lrb2(lt_scene* s, const lt_params* p, const lt_render_opts
   v = e ? LT_OK : use_copies(s, g, o, (char*)buf + lay.rep, lay.total - lay.rep, kp, st);
   if (v != LT_OK) return v;
   if (!e) e = launch_lrb2(dev_for(s, o), kp, o->attached != 0, s->has_dielectric, dI, buf, gp, L, st);
-  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp.rep, kp.rep_bits, s->n_mats, gp.d_albedo, st);
+  if (!e && kp.rep) e = launch_rep_sum(s->dev, kp, s->n_mats, gp, st);
   if (e) return fail(LT_ERR_CUDA, std::string("lt_backward_lrb2: ") + cudaGetErrorString(e));
   return LT_OK;
 }

@@ -51,9 +51,8 @@ cudaError_t launch_collect(const DevScene& S, const KParams& kp, const float* dI
   return LT_BY_WIDTH(S.width, launch_collect(S, kp, dI, tfloor, feats, targets, cap, count, L, st));
 }
 
-cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,
-                           cudaStream_t st) {
-  return w4::launch_rep_sum(S, rep, rep_bits, n_mats, d_albedo, st);
+cudaError_t launch_rep_sum(const DevScene& S, const KParams& kp, int n_mats, const GradPtrs& g, cudaStream_t st) {
+  return w4::launch_rep_sum(S, kp, n_mats, g, st);
 }
 
 cudaError_t launch_film_l2(const float* I, const float* T, int64_t n, float* dI, float* loss, int sms,

@@ -278,6 +278,30 @@ __device__ __forceinline__ void block_add3(float* dst, float3 v) {
   }
 }
 
+// The same over the passes of a call: the blocks of both passes add to `sum` (FP64), and `sum` is added
+// to dst once, by k_rep_sum or else (`last`) by the last block of the second pass.  Two thousand
+// blocks adding to one FP32 value, the signs of whose terms vary, left twice the rounding error of
+// one pass's (slab in box, 2^20 paths, relative to the sum of magnitudes: 2.4e-7 against 1.1e-7;
+// 7e-9 so).
+__device__ __forceinline__ void add_le_sum(float* dst, const double* sum) {
+  atomicAdd(dst, (float)__ldcg(sum)); atomicAdd(dst + 1, (float)__ldcg(sum + 1)); atomicAdd(dst + 2, (float)__ldcg(sum + 2));
+}
+__device__ __forceinline__ void block_add3(float* dst, float3 v, double* sum, bool last) {
+  __shared__ float sh[3][32];
+  v.x = warp_sum(v.x); v.y = warp_sum(v.y); v.z = warp_sum(v.z);
+  if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = v.x; sh[1][threadIdx.x >> 5] = v.y; sh[2][threadIdx.x >> 5] = v.z; }
+  __syncthreads();
+  if (threadIdx.x != 0 || !dst) return;
+  double a = v.x, b = v.y, c = v.z;
+  for (int w = 1; w < (int)((blockDim.x + 31) >> 5); ++w) { a += sh[0][w]; b += sh[1][w]; c += sh[2][w]; }
+  atomicAdd(sum, a); atomicAdd(sum + 1, b); atomicAdd(sum + 2, c);
+  if (!last) return;
+  __threadfence();
+  if (atomicAdd((unsigned long long*)(sum + 3), 1ull) + 1 != gridDim.x) return;
+  __threadfence();
+  add_le_sum(dst, sum);
+}
+
 // Gradient sink of a block: each parameter array that fits in shared memory (the host
 // decides per array) is accumulated there by the block (shared-memory atomics) and added to
 // the global array once at the end; the albedo and height arrays are small and every path
@@ -364,9 +388,10 @@ __device__ __forceinline__ void scatter_albedo_rep(float4* rep, int rep_bits, in
   }
 }
 // Add the copies up into the caller's array: a warp takes 256 consecutive entries (a texel has
-// eight copies at least), a lane eight of them.
+// eight copies at least), a lane eight of them; and the passes' sum of the emitted-radiance gradient.
 __global__ void __launch_bounds__(256) k_rep_sum(DevScene S, const float4* __restrict__ rep, int rep_bits, int n_mats,
-                                                 float* d_albedo) {
+                                                 float* d_albedo, const double* le_sum, float* d_Le) {
+  if (le_sum && d_Le && blockIdx.x == 0 && threadIdx.x == 0) add_le_sum(d_Le, le_sum);
   const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   const int mat = (int)(e >> rep_bits);
   const int4 m = mat < n_mats ? S.mat[mat] : make_int4(-1, 0, 0, 0);
@@ -1918,7 +1943,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
     atomicAdd(kp0.census + 4, (unsigned long long)nconns);
   }
   sink_end(kp0, g0, sgrad);
-  block_add3(g0.d_Le, gLe);
+  // le_sum is set with a path list, which both passes with known masks have
+  if (!LOCAL && MODE != 0 && MK && kp0.le_sum) block_add3(g0.d_Le, gLe, kp0.le_sum, MODE == 2 && !kp0.rep);
+  else block_add3(g0.d_Le, gLe);
 }
 
 template <bool ATT, bool ST, bool CH, bool FEW = false>
@@ -3327,10 +3354,9 @@ cudaError_t launch_bidir(const DevScene& S, const KParams& kp, const BidirArgs& 
   return cudaGetLastError();
 }
 
-cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,
-                           cudaStream_t st) {
-  const int64_t threads = ((int64_t)n_mats << rep_bits) / 8;
-  k_rep_sum<<<(int)((threads + 255) / 256), 256, 0, st>>>(S, rep, rep_bits, n_mats, d_albedo);
+cudaError_t launch_rep_sum(const DevScene& S, const KParams& kp, int n_mats, const GradPtrs& g, cudaStream_t st) {
+  const int64_t threads = ((int64_t)n_mats << kp.rep_bits) / 8;
+  k_rep_sum<<<(int)((threads + 255) / 256), 256, 0, st>>>(S, kp.rep, kp.rep_bits, n_mats, g.d_albedo, kp.le_sum, g.d_Le);
   return cudaGetLastError();
 }
 

@@ -50,6 +50,8 @@ struct KParams {
                                // primal with the LRB-3 state: [0] its 32-path chunks)
   uint32_t* multi;             // LRB-3 backward with a list: its paths with several connections
   unsigned long long* multi_n; // (k_lrb3_several appends, pass 2 visits), and their number
+  double* le_sum;              // zeroed: the passes' block sums of the emitted-radiance gradient (3), and
+                               // after them the blocks of pass 3 that are done (uint64); or null
   HitBits hits;                // primitives kept in the per-path records (bits 0: none)
   float4* rep;                 // LRB-3 pass 3: copies of the albedo gradient, [material][2^rep_bits]
   int rep_bits;                // (see scatter_albedo_rep), or null
@@ -125,9 +127,8 @@ struct BidirArgs {
   cudaError_t launch_collect(const DevScene& S, const KParams& kp, const float* dI, float tfloor, float* feats,   \
                              float* targets, int64_t cap, unsigned long long* count, const LaunchCfg& L,          \
                              cudaStream_t st);                                                                    \
-  /* sum of the copies of the albedo gradient, added to d_albedo (KParams::rep) */                                 \
-  cudaError_t launch_rep_sum(const DevScene& S, const float4* rep, int rep_bits, int n_mats, float* d_albedo,      \
-                             cudaStream_t st);                                                                     \
+  /* sum of the copies of the albedo gradient (KParams::rep), and of KParams::le_sum if there is one */            \
+  cudaError_t launch_rep_sum(const DevScene& S, const KParams& kp, int n_mats, const GradPtrs& g, cudaStream_t st); \
   cudaError_t launch_film_l2(const float* I, const float* T, int64_t n, float* dI, float* loss, int sms,          \
                              cudaStream_t st);                                                                    \
   cudaError_t launch_bidir(const DevScene& S, const KParams& kp, const BidirArgs& ba, bool backward, float* image, \
@@ -158,7 +159,8 @@ LT_KERNEL_LAUNCHERS
 //    lrb3_state_list), written by the plain primal so that passes 2 and 3 visit only those, and
 //    256 B of counters at lrb3_state_count: its length, the passes' counters of entries taken
 //    (two), the number of listed paths with several connections, the number of paths in the order
-//    (uint64 each); while the order is built, the list's place holds the paths' sort keys;
+//    (uint64 each), then KParams::le_sum; while the order is built, the list's place holds the
+//    paths' sort keys;
 //  - the order in which the plain primal takes the paths (uint32[n_paths] at lrb3_state_order;
 //    the backward reuses the array for the listed paths with several connections) and the
 //    counting sort's work area that builds it (kSortBins x kSortBlocks counts, then kSortBins
