@@ -1653,8 +1653,9 @@ __device__ __forceinline__ void lrb3_body(const DevScene& S0, const KParams& kp0
   // one at its own step, and short searches keep the warp's lanes together: pass 3 without known hits,
   // box 2^20 paths / slab 2^22, detached, 2 visits 2.02 / 1.14 ms, 3 1.83 / 1.06, 4 1.81 / 1.22, 6 2.21 / 1.49,
   // 10 2.64 / 1.57; both passes beyond their recorded hits, box 64 x 64 heights, 2^19 paths of depth 20 and
-  // 32, detached, 3 1.33 and 2.65, 5 1.54 and 3.00, 10 1.58 and 3.13, 20 1.59 and 3.21
-  constexpr int kBudget = MODE == 2 || (MODE == 1 && MK) ? 3 : kTraceBudget;
+  // 32, detached, 3 1.33 and 2.65, 5 1.54 and 3.00, 10 1.58 and 3.13, 20 1.59 and 3.21.  Batches keep the
+  // longer ones (small uneven scenes, passes 2 and 3: 3 visits 667 us, 10 632)
+  constexpr int kBudget = !BATCH && !LOCAL && (MODE == 2 || (MODE == 1 && MK)) ? 3 : kTraceBudget;
   HitWords<6> hw;  // the path's recorded primitives, valid below vertex hcap
   int hcap = 0;
   float c1[5];  // pass 2 without known masks: the first valid connection, for the record
